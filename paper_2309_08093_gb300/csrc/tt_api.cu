@@ -47,9 +47,7 @@ extern "C" int tt_sketch_unfold(tt_ctx* c, const void* A, const float* scales, i
   TT_TRY(tt_ensure_tables(c, sweep));
   if (c->det)  // fixed-point sketches of the requested modes (one scale for all)
     return tt_launch_unfold_det(c, A, scales, k == -1 ? (1u << c->d) - 1u : 1u << k, Y);
-  for (int kk = 0; kk < c->d; ++kk)
-    if (k == -1 || k == kk) TT_TRY(tt_launch_unfold(c, A, scales, kk, Y[kk]));
-  return TT_OK;
+  return k == -1 ? tt_launch_unfold_all(c, A, scales, Y) : tt_launch_unfold(c, A, scales, k, Y[k]);
 }
 
 extern "C" int tt_sketch_unfold_coo(tt_ctx* c, const int32_t* idx, const float* val, int64_t nnz, int k,
@@ -131,18 +129,13 @@ static int sweep_body(tt_ctx* c, const void* A, const float* scales, float* cons
     c->stream = c->side;
     c->in_sweep = true;
     int rc = TT_OK;
+    float* ys[TT_MAX_D];
+    for (int k = 0; k < d; ++k) ys[k] = c->d_Yall + c->yoff[k];
     if (c->det) {  // every mode in fixed point (one scale for all), Y_k's event as it is done
-      float* ys[TT_MAX_D];
-      for (int k = 0; k < d; ++k) ys[k] = c->d_Yall + c->yoff[k];
       rc = tt_launch_unfold_det(c, A, scales, (1u << d) - 1u, ys, c->ev_y);
       if (rc == TT_OK && !c->capture_mode) c->det_scale_reuse = true;
-    }
-    for (int k = 0; k < d && rc == TT_OK && !c->det; ++k) {
-      rc = tt_launch_unfold(c, A, scales, k, c->d_Yall + c->yoff[k]);
-      if (rc == TT_OK) {
-        const cudaError_t e = cudaEventRecord(c->ev_y[k], c->side);
-        if (e != cudaSuccess) rc = tt_cuda_check(c, e, "cudaEventRecord");
-      }
+    } else {
+      rc = tt_launch_unfold_all(c, A, scales, ys, c->ev_y);
     }
     c->stream = main_stream;
     c->in_sweep = false;

@@ -84,8 +84,19 @@ void tt_swap_draw(tt_ctx* c) {
     std::swap(c->d_ucount[k], o.ucount[k]);
     std::swap(c->rplan_valid[k], o.rplan_valid[k]);
   }
+  std::swap(c->d_hplan, o.hplan);
+  std::swap(c->d_rkey, o.rkey);
+  std::swap(c->d_tlist, o.tlist);
+  std::swap(c->d_tbucket, o.tbucket);
+  std::swap(c->pass_valid, o.pass_valid);
   std::swap(c->tables_valid, o.tables_valid);
   std::swap(c->tables_sweep, o.tables_sweep);
+}
+
+// new tables: the plans and the pattern built from the old ones are stale
+static void invalidate_plans(tt_ctx* c) {
+  for (int k = 0; k < TT_MAX_D; ++k) c->rplan_valid[k] = false;
+  c->pass_valid = false;
 }
 
 int tt_ensure_tables(tt_ctx* c, uint64_t sweep) {
@@ -98,7 +109,7 @@ int tt_ensure_tables(tt_ctx* c, uint64_t sweep) {
     k_gen_tables_dev<<<(int)((total + 255) / 256), 256, 0, c->stream>>>(
         c->seed, c->d_sweep_ptr, (c->flags & TT_FLAG_FIXED_SKETCH) ? 1 : 0, a, c->J, c->d_h, c->d_v);
     TT_LAUNCH(c, "k_gen_tables_dev");
-    for (int k = 0; k < TT_MAX_D; ++k) c->rplan_valid[k] = false;
+    invalidate_plans(c);
     return TT_OK;
   }
   if (c->flags & TT_FLAG_FIXED_SKETCH) sweep = 0;
@@ -119,7 +130,7 @@ int tt_ensure_tables(tt_ctx* c, uint64_t sweep) {
   TT_LAUNCH(c, "k_gen_tables");
   c->tables_valid = true;
   c->tables_sweep = sweep;
-  for (int k = 0; k < TT_MAX_D; ++k) c->rplan_valid[k] = false;
+  invalidate_plans(c);
   return TT_OK;
 }
 
@@ -208,6 +219,7 @@ struct RPlanOut {
   int64_t* ustart[TT_MAX_D];
   int32_t* ucount[TT_MAX_D];
   uint32_t* plan[TT_MAX_D];
+  int32_t* key[TT_MAX_D];  // c of each plan entry (null: not wanted)
 };
 
 __device__ __forceinline__ int plan_mode(const RPlanAll& P) {
@@ -313,6 +325,7 @@ __global__ void k_rplan_scatter(RPlanAll P, const int32_t* h, const int8_t* v, c
   int32_t* cursor = cursor_all + (int64_t)m * a.J;
   const int64_t* off = off_all + (int64_t)m * (a.J + 1);
   uint32_t* plan = o.plan[m];
+  int32_t* keys = o.key[m];
   RestWalker wk;
   wk.init(a, r0 + threadIdx.x, blockDim.x);
   if (P.direct[m]) {
@@ -320,8 +333,9 @@ __global__ void k_rplan_scatter(RPlanAll P, const int32_t* h, const int8_t* v, c
       int key, neg;
       int64_t ofs;
       wk.entry(a, h, v, &key, &neg, &ofs);
-      const int pos = atomicAdd(&cursor[key], 1);
-      plan[off[key] + pos] = (uint32_t)ofs | ((uint32_t)neg << 31);
+      const int64_t pos = off[key] + atomicAdd(&cursor[key], 1);
+      plan[pos] = (uint32_t)ofs | ((uint32_t)neg << 31);
+      if (keys) keys[pos] = key;
     }
     return;
   }
@@ -342,8 +356,9 @@ __global__ void k_rplan_scatter(RPlanAll P, const int32_t* h, const int8_t* v, c
     int key, neg;
     int64_t ofs;
     wk.entry(a, h, v, &key, &neg, &ofs);
-    const int pos = atomicAdd(&hist[key], 1);
-    plan[off[key] + pos] = (uint32_t)ofs | ((uint32_t)neg << 31);  // fibre index | sign
+    const int64_t pos = off[key] + atomicAdd(&hist[key], 1);
+    plan[pos] = (uint32_t)ofs | ((uint32_t)neg << 31);  // fibre index | sign
+    if (keys) keys[pos] = key;
   }
 }
 
@@ -486,16 +501,15 @@ __global__ void __launch_bounds__(32) k_rplan_dscatter(DPlan D, int d, int J, co
   }
 }
 
-// Plans of every mode for the current tables. In graph-capture mode with per-sweep draws the
-// plans are rebuilt at the sweep's first data sketch (mode 0) and reused by the other modes.
-int tt_ensure_rplan(tt_ctx* c, int k) {
-  const bool redraw = c->capture_mode && !(c->flags & TT_FLAG_FIXED_SKETCH) && !c->user_tables;
-  if (redraw ? k != 0 : c->rplan_valid[k]) return TT_OK;
+// Plans of the modes in `mask` for the current tables, built together.
+static int build_plans(tt_ctx* c, unsigned mask) {
   RPlanAll P;
   RPlanOut o;
-  P.d = c->d;
+  int nm = 0;
   P.bstart[0] = 0;
-  for (int m = 0; m < c->d; ++m) {
+  for (int k = 0; k < c->d; ++k) {
+    if (!(mask & (1u << k))) continue;
+    const int m = nm++;
     RPlanArgs& a = P.m[m];
     for (int s = 0; s < c->d; ++s) {
       a.n[s] = c->n[s];
@@ -504,32 +518,34 @@ int tt_ensure_rplan(tt_ctx* c, int k) {
     }
     for (int s = 0; s <= c->d; ++s) a.noff[s] = c->noff[s];
     a.d = c->d;
-    a.k = m;
+    a.k = k;
     a.J = c->J;
-    a.R = c->R[m];
+    a.R = c->R[k];
     P.direct[m] = a.R <= 8 * (int64_t)c->J;
     P.pb[m] = P.direct[m] ? 1024
                           : (int)std::max<int64_t>((int64_t)c->J, std::min<int64_t>(TT_PLAN_BLOCK, (a.R + 303) / 304));
     P.bstart[m + 1] = P.bstart[m] + std::max<int64_t>(1, (a.R + P.pb[m] - 1) / P.pb[m]);
-    o.ulist[m] = c->d_ulist[m];
-    o.ustart[m] = c->d_ustart[m];
-    o.ucount[m] = c->d_ucount[m];
-    o.plan[m] = c->d_rplan[m];
+    o.ulist[m] = c->d_ulist[k];
+    o.ustart[m] = c->d_ustart[k];
+    o.ucount[m] = c->d_ucount[k];
+    o.plan[m] = c->d_rplan[k];
+    o.key[m] = k == 1 && c->pass_head && !c->head_sorted ? c->d_rkey : nullptr;
   }
+  P.d = nm;
   int32_t* count = c->d_plan0_cursor;
   if (c->spare_pending && c->stream != c->side) TT_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_spare, 0));
-  TT_CUDA(c, cudaMemsetAsync(count, 0, sizeof(int32_t) * c->J * c->d, c->stream));
+  TT_CUDA(c, cudaMemsetAsync(count, 0, sizeof(int32_t) * c->J * nm, c->stream));
   const size_t hsm = sizeof(int) * c->J;
   if (hsm > 48 * 1024) {
     TT_CUDA(c, cudaFuncSetAttribute(k_rplan_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm));
     TT_CUDA(c, cudaFuncSetAttribute(k_rplan_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm));
   }
-  const int blocks = (int)P.bstart[c->d];
+  const int blocks = (int)P.bstart[nm];
   k_rplan_count<<<blocks, 512, hsm, c->stream>>>(P, c->d_h, c->d_v, count);
   TT_LAUNCH(c, "k_rplan_count");
-  k_rplan_scan<<<c->d, 1024, 0, c->stream>>>(c->J, count, c->d_rtmp, o);
+  k_rplan_scan<<<nm, 1024, 0, c->stream>>>(c->J, count, c->d_rtmp, o);
   TT_LAUNCH(c, "k_rplan_scan");
-  if (c->det) {  // fibres of each group in index order
+  if (c->det) {  // fibres of each group in index order (every mode: positions are modes)
     DPlan D;
     D.bstart[0] = 0;
     int64_t roff = 0;
@@ -555,9 +571,35 @@ int tt_ensure_rplan(tt_ctx* c, int k) {
     k_rplan_scatter<<<blocks, 512, hsm, c->stream>>>(P, c->d_h, c->d_v, c->d_rtmp, count, o);
     TT_LAUNCH(c, "k_rplan_scatter");
   }
-  for (int m = 0; m < c->d; ++m) c->rplan_valid[m] = true;
+  for (int k = 0; k < c->d; ++k)
+    if (mask & (1u << k)) c->rplan_valid[k] = true;
   return TT_OK;
 }
+
+// In graph-capture mode with per-sweep draws everything is rebuilt at the sweep's data sketches.
+static bool redraw(const tt_ctx* c) {
+  return c->capture_mode && !(c->flags & TT_FLAG_FIXED_SKETCH) && !c->user_tables;
+}
+
+int tt_ensure_plans(tt_ctx* c, unsigned mask, bool pass) {
+  unsigned need = 0;
+  for (int k = 0; k < c->d; ++k)
+    if ((mask & (1u << k)) && (redraw(c) || !c->rplan_valid[k])) need |= 1u << k;
+  if (need) TT_TRY(build_plans(c, need));
+  if (pass && (redraw(c) || !c->pass_valid)) {
+    if (c->spare_pending && c->stream != c->side) TT_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_spare, 0));
+    TT_TRY(tt_launch_pass_plans(c));
+    c->pass_valid = true;
+  }
+  return TT_OK;
+}
+
+// Plan of mode k, and of all modes with it (in graph-capture mode at the sweep's first data sketch).
+int tt_ensure_rplan(tt_ctx* c, int k) {
+  if (redraw(c) ? k != 0 : c->rplan_valid[k]) return TT_OK;
+  return build_plans(c, (1u << c->d) - 1u);
+}
+
 
 int tt_ensure_plan0(tt_ctx* c) { return tt_ensure_rplan(c, 0); }
 
@@ -565,14 +607,16 @@ int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep) {
   // (the deterministic mode's plans too: tt_ensure_rplan builds them in index order)
   if (c->capture_mode || c->user_tables || (c->flags & TT_FLAG_FIXED_SKETCH)) return TT_OK;
   bool ready = c->spare.tables_valid && c->spare.tables_sweep == sweep;
-  for (int k = 0; k < c->d; ++k) ready = ready && c->spare.rplan_valid[k];
+  const unsigned plans = tt_pass_plans(c);
+  for (int k = 0; k < c->d; ++k) ready = ready && (c->spare.rplan_valid[k] || !(plans & (1u << k)));
+  ready = ready && (c->spare.pass_valid || c->det);
   if (ready) return TT_OK;
   tt_swap_draw(c);  // build into the spare through the current-draw fields
   cudaStream_t s0 = c->stream;
   c->stream = c->side;
   c->tables_valid = false;
   int rc = tt_ensure_tables(c, sweep);
-  if (rc == TT_OK) rc = tt_ensure_rplan(c, 0);
+  if (rc == TT_OK) rc = tt_ensure_plans(c, plans, !c->det);
   cudaError_t e = cudaEventRecord(c->ev_spare, c->side);
   c->stream = s0;
   tt_swap_draw(c);
@@ -589,30 +633,9 @@ int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep) {
 // lifetime
 
 static void free_all(tt_ctx* c) {
-  void* ps[] = {c->d_h, c->d_v, c->d_plan0, c->d_plan0_off, c->d_plan0_cursor, c->d_ghat,
-                c->d_twiddle, c->d_twstage, c->d_suffix, c->d_prefix, c->d_prefix_tmp, c->d_SH, c->d_Y,
-                c->d_gram, c->d_core_old, c->d_changes, c->d_status, c->d_err_acc, c->d_errs, c->d_ws_acc, c->d_rint, c->d_slab_u, c->d_Yall, c->d_xgram, c->d_gram64,
-                c->d_det_misc, c->d_y64, c->d_gram_part, c->d_part_err, c->d_part_chg, c->d_det_bcnt, c->d_det_kv};
-  for (void* p : ps)
-    if (p) cudaFree(p);
+  if (c->ws_block) cudaFree(c->ws_block);
   tt_host_free(c);
-  void* sp[] = {c->spare.h, c->spare.v};
-  for (void* p : sp)
-    if (p) cudaFree(p);
   if (c->ev_spare) cudaEventDestroy(c->ev_spare);
-  for (int k = 0; k < TT_MAX_D; ++k) {
-    if (c->spare.rplan[k]) cudaFree(c->spare.rplan[k]);
-    if (c->spare.ulist[k]) cudaFree(c->spare.ulist[k]);
-    if (c->spare.ustart[k]) cudaFree(c->spare.ustart[k]);
-    if (c->spare.ucount[k]) cudaFree(c->spare.ucount[k]);
-  }
-  for (int k = 0; k < TT_MAX_D; ++k) {
-    if (c->d_rplan[k]) cudaFree(c->d_rplan[k]);
-    if (c->d_ulist[k]) cudaFree(c->d_ulist[k]);
-    if (c->d_ustart[k]) cudaFree(c->d_ustart[k]);
-    if (c->d_ucount[k]) cudaFree(c->d_ucount[k]);
-  }
-  if (c->d_rtmp) cudaFree(c->d_rtmp);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   for (int k = 0; k < TT_MAX_D; ++k)
@@ -623,9 +646,9 @@ static void free_all(tt_ctx* c) {
   if (c->ev_out) cudaEventDestroy(c->ev_out);
 }
 
-// Every device workspace of a context, in allocation order: f(&pointer, bytes). Used twice by
-// tt_sketch_init: to sum the sizes (the cap of tt_set_workspace_limit is checked before any CUDA
-// call) and to allocate. Fills the size bookkeeping of the context (R, yoff, changes_cap,
+// Every device workspace of a context, in order: f(&pointer, bytes). Used twice by tt_sketch_init: to
+// sum the sizes (the cap of tt_set_workspace_limit is checked before any CUDA call) and to cut the
+// one allocation up. Fills the size bookkeeping of the context (R, yoff, changes_cap,
 // rint_r1p) as it goes.
 template <typename F>
 static void tt_workspace_each(tt_ctx* c, F&& A) {
@@ -660,6 +683,23 @@ static void tt_workspace_each(tt_ctx* c, F&& A) {
   A((void**)&c->d_Yall, sizeof(float) * c->yoff[c->d]);
   A((void**)&c->d_gram, sizeof(float) * (c->smax + c->nmax) * c->smax);
   if (c->solve64) A((void**)&c->d_gram64, sizeof(double) * (c->smax + c->nmax) * c->smax);
+  if (c->pass_head) {
+    if (c->head_sorted) {
+      A((void**)&c->d_hplan, sizeof(uint32_t) * c->R[1]);
+      A((void**)&c->spare.hplan, sizeof(uint32_t) * c->R[1]);
+    }
+    A((void**)&c->d_rkey, sizeof(int32_t) * c->R[1]);
+    A((void**)&c->spare.rkey, sizeof(int32_t) * c->R[1]);
+    A((void**)&c->d_y01, sizeof(float) * c->J * (size_t)(c->p0 + c->p1));
+  }
+  if (c->pass_tail) {
+    const size_t e = sizeof(uint16_t) * 4 * (size_t)c->tail_blocks * c->tail_nchunk;
+    const size_t b = sizeof(uint32_t) * (size_t)(c->J + (c->tail_chunk + 31) / 32) * c->tail_nchunk;
+    A((void**)&c->d_tlist, e);
+    A((void**)&c->d_tbucket, b);
+    A((void**)&c->spare.tlist, e);
+    A((void**)&c->spare.tbucket, b);
+  }
   if (c->det) {
     A((void**)&c->d_det_misc, sizeof(int) * 4);
     A((void**)&c->d_y64, sizeof(int64_t) * c->yoff[c->d]);
@@ -688,8 +728,7 @@ static void tt_workspace_each(tt_ctx* c, F&& A) {
 
 static std::atomic<uint64_t> g_workspace_limit{0};
 
-// Total bytes of the workspaces above (each allocation rounded up to the 16 bytes cudaMalloc is
-// given at least); touches no device.
+// Total bytes of the workspaces above (each rounded up to 256 bytes); touches no device.
 static uint64_t tt_workspace_plan(tt_ctx* c) {
   uint64_t total = 0;
   tt_workspace_each(c, [&](void**, size_t bytes) { total += (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255; });
@@ -777,19 +816,29 @@ extern "C" int tt_sketch_init(tt_ctx** out, const tt_params* p, void* stream) {
 
   // The workspaces are planned (sizes summed) before anything is allocated, so that a process-wide
   // cap (tt_set_workspace_limit) is enforced before any CUDA call.
-  const uint64_t planned = tt_workspace_plan(c);
-  c->ws_bytes = planned;
+  tt_pass_plan(c);
+  uint64_t planned = tt_workspace_plan(c);
   const uint64_t cap = g_workspace_limit.load();
+  if (cap && planned > cap && (c->pass_head || c->pass_tail)) {  // one launch per mode needs less
+    c->pass_head = c->pass_tail = c->head_sorted = false;
+    c->tail_modes = 0;
+    planned = tt_workspace_plan(c);
+  }
+  c->ws_bytes = planned;
   if (cap && planned > cap) {
     fprintf(stderr, "tt_sketch_init: workspaces need %llu bytes, above the limit of %llu bytes\n",
             (unsigned long long)planned, (unsigned long long)cap);
     delete c;
     return TT_ENOMEM;
   }
-  cudaError_t e = cudaSuccess;
-  tt_workspace_each(c, [&](void** ptr, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(ptr, std::max<size_t>(bytes, 16));
-  });
+  // one allocation, cut into the workspaces on 256-byte boundaries as tt_workspace_plan counts them
+  cudaError_t e = cudaMalloc(&c->ws_block, planned);
+  char* at = static_cast<char*>(c->ws_block);
+  if (e == cudaSuccess)
+    tt_workspace_each(c, [&](void** ptr, size_t bytes) {
+      *ptr = at;
+      at += (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255;
+    });
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
   if (e == cudaSuccess) {
     int least = 0, greatest = 0;
@@ -830,6 +879,8 @@ extern "C" int tt_sketch_init(tt_ctx** out, const tt_params* p, void* stream) {
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c->d_twstage, tws.data(), sizeof(float2) * tws.size(), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
+  if (e == cudaSuccess && c->d_y01)
+    e = cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)c->J * (c->p0 + c->p1), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
     free_all(c);
@@ -877,6 +928,6 @@ extern "C" int tt_sketch_set_tables(tt_ctx* c, const int32_t* h_host, const int8
   c->user_tables = true;
   c->spare.tables_valid = false;
   c->tables_valid = true;
-  for (int k = 0; k < TT_MAX_D; ++k) c->rplan_valid[k] = false;
+  invalidate_plans(c);
   return TT_OK;
 }

@@ -76,6 +76,11 @@ struct TtDraw {
   int32_t* ulist[TT_MAX_D] = {nullptr};
   int64_t* ustart[TT_MAX_D] = {nullptr};
   int32_t* ucount[TT_MAX_D] = {nullptr};
+  uint32_t* hplan = nullptr;
+  int32_t* rkey = nullptr;
+  uint16_t* tlist = nullptr;
+  uint32_t* tbucket = nullptr;
+  bool pass_valid = false;
   bool tables_valid = false;
   uint64_t tables_sweep = 0;
   bool rplan_valid[TT_MAX_D] = {false};
@@ -124,7 +129,21 @@ struct tt_ctx {
   int32_t* d_ucount[TT_MAX_D] = {nullptr};  // number of distinct c values (device scalar)
   int64_t* d_rtmp = nullptr;                 // d x (J + 1) bucket offsets of the plan build
   bool rplan_valid[TT_MAX_D] = {false};
-  float* d_Ypart = nullptr;                  // unused placeholder
+  // data sketches of several modes from one read of A (tt_pass.cu): the head pass covers modes 0
+  // and 1, the tail pass the last tail_modes (1 or 2) modes; set from the shape by tt_pass_plan
+  bool pass_head = false, pass_tail = false;
+  int tail_modes = 0;
+  int tail_chunk = 0, tail_nchunk = 0;  // entries per chunk of a tail-pass slab, chunks
+  int tail_blocks = 0;                  // list blocks per chunk, at most
+  int p0 = 0, p1 = 0;                   // row lengths of the head pass's accumulators (n_0, n_1 up to 4s)
+  bool head_sorted = false;             // the head pass's slabs are sorted by k_pass_plans (else mode 1's plan)
+  uint32_t* d_hplan = nullptr;          // head pass: slabs by c (when head_sorted)
+  int32_t* d_rkey = nullptr;            // head pass: c of each slab of its plan
+  uint16_t* d_tlist = nullptr;          // tail pass: the head's entries by bucket, chunk after chunk
+  uint32_t* d_tbucket = nullptr;        // tail pass: bucket words (J per chunk), then sign words
+  bool pass_valid = false;              // d_hplan, d_tlist, d_tbucket are those of the current draw
+  float* d_y01 = nullptr;               // J x p0 then J x p1: Y_0 and Y_1 by rows (zero between head passes)
+  bool y01_zero = true;                 // they are (false after a launch that failed in between)
   TtDraw spare;                              // the next sweep's draw (see TtDraw)
   cudaEvent_t ev_spare = nullptr;            // end of the spare's build on `side`
   bool spare_pending = false;
@@ -210,6 +229,7 @@ struct tt_ctx {
   int tune_seg_mult[TT_MAX_D] = {0};   // multiplier of the work-item count
   int tune_cta_per_sm[TT_MAX_D] = {0}; // CTAs per SM (1 or 2)
 
+  void* ws_block = nullptr;     // the one device allocation that holds every workspace
   uint64_t ws_bytes = 0;        // bytes of the workspaces planned at creation (tt_workspace_each)
 
   // host-buffer entry points (tt_host.cu, allocated on first use): two staging buffers for the
@@ -284,9 +304,19 @@ int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep);
 void tt_swap_draw(tt_ctx* c);
 int tt_ensure_plan0(tt_ctx* c);
 int tt_ensure_rplan(tt_ctx* c, int k);
+// the plans of the modes in `mask`, and those of the passes
+int tt_ensure_plans(tt_ctx* c, unsigned mask, bool pass);
 
 // kernels' host entry points (one translation unit each)
 int tt_launch_unfold(tt_ctx* c, const void* A, const float* scales, int k, float* Y);
+int tt_launch_unfold_planned(tt_ctx* c, const void* A, const float* scales, int k, float* Y);  // its plan is built
+// data sketches of every mode (tt_pass.cu): passes over A that serve two modes each where the shape
+// allows, tt_launch_unfold for the other modes; ev[k] (optional) is recorded after Y[k]
+int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev = nullptr);
+void tt_pass_plan(tt_ctx* c);                 // which modes the passes cover, from the shape
+unsigned tt_pass_mask(const tt_ctx* c);       // modes covered by the passes
+unsigned tt_pass_plans(const tt_ctx* c);      // modes whose fibre plan tt_launch_unfold_all reads
+int tt_launch_pass_plans(tt_ctx* c);          // d_hplan, d_rkey, d_tlist, d_tbucket of the current draw
 int tt_launch_unfold_coo(tt_ctx* c, const int32_t* idx, const float* val, int64_t nnz, int k, float* const* Y);
 // d_err_acc[0..2] = sum val^2, sum val X(i), ||X||^2 of a sparse tensor in coordinate form
 int tt_launch_rel_error_coo(tt_ctx* c, const int32_t* idx, const float* val, int64_t nnz, float* const* cores);

@@ -1,0 +1,911 @@
+// Part (a) for several modes from one read of A (Alg. 1, Eqs. (eqn_h), (eqn_v)). With the modes cut
+// into a head (the first ones) and a tail (the others), A is a list of contiguous slabs, one per
+// tail index t, and the definition of Y_k regroups in two ways:
+//
+// k_head_pass, modes 0 and 1 (head = modes 0, 1; slab n_0 x n_1). With c_t the hash of the tail
+// modes, Z_c = sum over the slabs with c_t = c of sign_t * slab, and
+//     Y_0[(c + h_1(i_1)) mod J, i_0] += v_1(i_1) Z_c[i_0, i_1],
+//     Y_1[(c + h_0(i_0)) mod J, i_1] += v_0(i_0) Z_c[i_0, i_1].
+// A CTA walks slabs in the order of c (the plan of mode 1), sums a run of equal c in registers and
+// adds each finished run to both sketches: one read of A where one launch per mode took two.
+//
+// k_tail_pass, the last one or two modes (head = the modes before them). With q_t the CountSketch of
+// slab t under the head's hashes (J buckets, the same pattern for every slab) the tail modes s, l give
+//     Y_l[(c + h_s(i_s)) mod J, i_l] += v_s(i_s) q_t[c],   Y_s[(c + h_l(i_l)) mod J, i_s] += v_l(i_l) q_t[c],
+// again one read of A for both. The modes between (d >= 5) keep one launch each (tt_unfold.cu).
+#include <algorithm>
+#include <type_traits>
+
+#include "tt_unfold.cuh"
+
+namespace {
+
+__device__ __forceinline__ void red4(float* p, float4 v) { atomicAdd(reinterpret_cast<float4*>(p), v); }
+
+// ---------------------------------------------------------------------------------------------
+// head pass
+
+struct HeadArgs {
+  const char* A;
+  const float* scales;
+  const uint32_t* plan;  // slabs grouped by c: fibre index of the slab | sign in bit 31
+  const int32_t* key;    // c of each plan entry
+  const int32_t *h0, *h1;
+  const int8_t *v0, *v1;
+  float* Y0r;  // J x p0, row b = bucket b of Y_0
+  float* Y1r;  // J x p1, row b = bucket b of Y_1
+  int64_t R;   // slabs
+  int J, n0, n1, p0, p1;
+  int G1, nch;  // columns i_1 per chunk of a slab, chunks
+  int nseg;     // segments of the plan
+  int pitch;    // floats per column of the transposition tile (a multiple of 32)
+  uint32_t inv_n0;  // 2^32 / n_0 rounded up
+  float* zero[2];   // sketches of the tail pass (which follows): zeroed on the side
+  int64_t nzero[2];
+};
+constexpr int HEAD_BATCH = 256;  // plan entries staged at a time
+constexpr int HEAD_TMAX = 320;   // two CTAs per SM at 102 registers
+// entries of a slab's chunk per thread
+template <int DT>
+constexpr int head_acc() { return DT == TT_F64 ? 16 : 32; }
+
+// 16-byte words [v ^ (i_1 / 4 mod 8)] of column i_1: with a pitch of 32 floats the 16-byte stores of
+// a column and the reads below (8 column groups x 4 consecutive rows) both touch every bank once
+__device__ __forceinline__ int tile_at(int i1, int i0, int pitch) {
+  return i1 * pitch + ((((i0 >> 2) ^ ((i1 >> 2) & 7)) << 2) | (i0 & 3));
+}
+
+// VB bytes of A as 32-bit words
+template <int VB>
+__device__ __forceinline__ void head_load(const char* p, uint32_t* r) {
+  if constexpr (VB == 16) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    r[0] = u.x, r[1] = u.y, r[2] = u.z, r[3] = u.w;
+  } else if constexpr (VB == 8) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    r[0] = u.x, r[1] = u.y;
+  } else if constexpr (VB == 4) {
+    r[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+  } else if constexpr (VB == 2) {
+    r[0] = __ldg(reinterpret_cast<const unsigned short*>(p));
+  } else {
+    r[0] = __ldg(reinterpret_cast<const unsigned char*>(p));
+  }
+}
+
+// acc[e] += s * entry e of the loaded words (s = +-1)
+template <int DT, int EPV>
+__device__ __forceinline__ void head_add(const uint32_t* w, float s, float* acc) {
+  if constexpr (DT == TT_F32 && EPV > 1) {
+#pragma unroll
+    for (int e = 0; e < EPV; e += 2) {
+      const float2 d = tt_ffma2(make_float2(s, s), make_float2(__uint_as_float(w[e]), __uint_as_float(w[e + 1])),
+                                make_float2(acc[e], acc[e + 1]));
+      acc[e] = d.x, acc[e + 1] = d.y;
+    }
+  } else if constexpr (DT == TT_F32) {
+    acc[0] = fmaf(s, __uint_as_float(w[0]), acc[0]);
+  } else if constexpr (DT == TT_F64) {
+#pragma unroll
+    for (int e = 0; e < EPV; ++e) {
+      const unsigned long long b = ((unsigned long long)w[2 * e + 1] << 32) | w[2 * e];
+      acc[e] = fmaf(s, (float)__longlong_as_double((long long)b), acc[e]);
+    }
+  } else if constexpr (DT == TT_BF16) {
+    const unsigned short sb = tt_bf16_sign(s);
+    if constexpr (EPV == 1) {
+      acc[0] = tt_fma_bf16((unsigned short)w[0], sb, acc[0]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < EPV; e += 2) tt_fma_bf16x2(w[e >> 1], sb, acc[e], acc[e + 1]);
+    }
+  } else {
+    const unsigned short sh = tt_f16_sign(s);
+    if constexpr (EPV == 1) {
+      acc[0] = tt_fma_e4m3((unsigned short)w[0], sh, acc[0]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < EPV; e += 4) tt_fma_e4m3x4(w[e >> 2], sh, acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+    }
+  }
+}
+
+// Bound: DRAM while runs are long (100^4 FP32, J = 1024, 9.8 slabs per run: 80 us, 5.0 TB/s), the
+// flushes' L2 atomics and tile traffic beside it when they are short (J = 4096, 2.4 slabs per run:
+// 113 us for both modes, 206 us with one launch per mode). The flushes go to L2 as 16-byte atomic adds
+// along rows (5.9 TB/s of sums, measured alone) because shared-memory float atomics at random
+// buckets sustain half of that (0.75 T adds/s) and need a copy of the columns per CTA. Two CTAs per
+// SM: one flushes while the other loads.
+// A slab's chunk is read as a run of VB-byte vectors, whatever columns they lie in: thread t holds
+// the vectors t + T j. U slabs are loaded ahead of the sums.
+template <int DT, int VB>
+__global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
+  constexpr int EB = TtElem<DT>::bytes;
+  constexpr int EPV = VB / EB;                // entries per vector
+  constexpr int NV = head_acc<DT>() / EPV;    // vectors per thread
+  constexpr int W = VB < 4 ? 1 : VB / 4;      // registers per vector
+  constexpr int U = NV * W >= 32 ? 1 : 32 / (NV * W);
+  extern __shared__ __align__(16) float hsm[];
+  const int T = blockDim.x, t = threadIdx.x;
+  for (int z = 0; z < 2; ++z)
+    for (int64_t i = (int64_t)blockIdx.x * T + t; i < a.nzero[z]; i += (int64_t)gridDim.x * T) a.zero[z][i] = 0.f;
+  const int n0 = a.n0, J = a.J, pitch = a.pitch;
+  const int ch = blockIdx.x % a.nch, seg = blockIdx.x / a.nch;
+  const int c0 = ch * a.G1, g1 = min(a.G1, a.n1 - c0), g1p = (g1 + 3) & ~3;
+  const int rows_tile = (a.G1 + 3) & ~3, n0p = (n0 + 3) & ~3;
+  float* tile = hsm;                                        // rows_tile x pitch
+  float* cf0 = tile + (size_t)rows_tile * pitch;            // n0p: v_0 (times the FP8 scale)
+  float* sc0 = cf0 + n0p;                                   // n0p: FP8 scale (1 otherwise)
+  int* hh0 = reinterpret_cast<int*>(sc0 + n0p);             // n0p
+  int* hh1 = hh0 + n0p;                                     // rows_tile: h_1, sign in bit 31
+  uint32_t* sw = reinterpret_cast<uint32_t*>(hh1 + rows_tile);  // HEAD_BATCH
+  int* sk = reinterpret_cast<int*>(sw + HEAD_BATCH);        // HEAD_BATCH
+  for (int i = t; i < n0p; i += T) {
+    const float s = a.scales && i < n0 ? __ldg(a.scales + i) : 1.f;
+    sc0[i] = s;
+    cf0[i] = i < n0 && __ldg(a.v0 + i) < 0 ? -s : s;
+    hh0[i] = i < n0 ? __ldg(a.h0 + i) : 0;
+  }
+  for (int i = t; i < g1; i += T) hh1[i] = __ldg(a.h1 + c0 + i) | (__ldg(a.v1 + c0 + i) < 0 ? (int)0x80000000 : 0);
+  for (int i = t; i < rows_tile * pitch; i += T) tile[i] = 0.f;  // the padding stays zero
+  const int64_t eb = a.R * seg / a.nseg, ee = a.R * (seg + 1) / a.nseg;
+  const int ne = n0 * g1;  // entries of a slab's chunk
+  const char* base = a.A + (int64_t)c0 * n0 * EB + (int64_t)t * VB;
+  const int64_t fb = (int64_t)n0 * EB;
+  const bool quads = EPV >= 4 && (n0 & 3) == 0;  // every four entries lie in one column
+  float acc[NV][EPV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j)
+#pragma unroll
+    for (int e = 0; e < EPV; ++e) acc[j][e] = 0.f;
+
+  // the finished run of group c: rows of Y_0 and Y_1 (16-byte atomic adds), through the tile where a
+  // thread's entries are not a row's
+  auto flush = [&](int c) {
+    __syncthreads();  // the tile's last readers are done
+    if (quads) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j)
+#pragma unroll
+        for (int e = 0; e + 3 < EPV; e += 4) {
+            const int en = (t + T * j) * EPV + e;
+            if (en < ne) {
+              const int i1 = (int)__umulhi((uint32_t)en, a.inv_n0), i0 = en - i1 * n0;
+              const int hw = hh1[i1];
+              const float s1 = hw < 0 ? -1.f : 1.f;
+              const float4 z = make_float4(acc[j][e], acc[j][e + 1], acc[j][e + 2], acc[j][e + 3]);
+              *reinterpret_cast<float4*>(tile + tile_at(i1, i0, pitch)) = z;
+              float4 m = make_float4(s1 * z.x, s1 * z.y, s1 * z.z, s1 * z.w);
+              if (DT == TT_FP8E4M3) m.x *= sc0[i0], m.y *= sc0[i0 + 1], m.z *= sc0[i0 + 2], m.w *= sc0[i0 + 3];
+              red4(a.Y0r + (int64_t)tt_modj(c + (hw & 0x7FFFFFFF), J) * a.p0 + i0, m);
+            }
+          }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NV; ++j)
+#pragma unroll
+        for (int e = 0; e < EPV; ++e) {
+          const int en = (t + T * j) * EPV + e;
+          if (en < ne) {
+            const int i1 = (int)__umulhi((uint32_t)en, a.inv_n0), i0 = en - i1 * n0;
+            tile[tile_at(i1, i0, pitch)] = acc[j][e];
+          }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+#pragma unroll
+      for (int e = 0; e < EPV; ++e) acc[j][e] = 0.f;
+    __syncthreads();
+    // the columns of the tile as rows of Y_1: 4 rows i_0 x 32 columns i_1 per warp step
+    const int g = t & 7, q = (t >> 3) & 3;
+    const int nq = n0p >> 2, ng = (g1p + 31) >> 5;
+    for (int task = t >> 5; task < nq * ng; task += T >> 5) {
+      const int ig = task / nq, i0 = 4 * (task - ig * nq) + q, i1 = 32 * ig + 4 * g;
+      if (i0 < n0 && i1 < g1p) {
+        const float* src = tile + tile_at(i1, i0, pitch);  // columns i1 .. i1 + 3 share the swizzle
+        const float s = cf0[i0];
+        red4(a.Y1r + (int64_t)tt_modj(c + hh0[i0], J) * a.p1 + c0 + i1,
+             make_float4(s * src[0], s * src[pitch], s * src[2 * pitch], s * src[3 * pitch]));
+      }
+    }
+    if (!quads)  // and the rows of Y_0
+      for (int i = t; i < nq * g1; i += T) {
+        const int i1 = i / nq, i0 = 4 * (i - i1 * nq);
+        const int hw = hh1[i1];
+        const float s1 = hw < 0 ? -1.f : 1.f;
+        const float4 z = *reinterpret_cast<const float4*>(tile + tile_at(i1, i0, pitch));
+        float4 m = make_float4(s1 * z.x, s1 * z.y, s1 * z.z, s1 * z.w);
+        if (DT == TT_FP8E4M3) m.x *= sc0[i0], m.y *= sc0[i0 + 1], m.z *= sc0[i0 + 2], m.w *= sc0[i0 + 3];
+        red4(a.Y0r + (int64_t)tt_modj(c + (hw & 0x7FFFFFFF), J) * a.p0 + i0, m);
+      }
+  };
+
+  int cur = -1;
+  for (int64_t b0 = eb; b0 < ee; b0 += HEAD_BATCH) {
+    const int nb = (int)min((int64_t)HEAD_BATCH, ee - b0);
+    __syncthreads();
+    for (int i = t; i < nb; i += T) {
+      sw[i] = __ldg(a.plan + b0 + i);
+      sk[i] = __ldg(a.key + b0 + i);
+    }
+    __syncthreads();
+    for (int i = 0; i < nb; i += U) {
+      uint32_t r[U][NV][W];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (U == 1 || i + u < nb) {
+          const char* p = base + (int64_t)(sw[i + u] & 0x7FFFFFFFu) * fb;
+#pragma unroll
+          for (int j = 0; j < NV; ++j)
+            if ((t + T * j) * EPV < ne) head_load<VB>(p + T * j * VB, r[u][j]);
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (U == 1 || i + u < nb) {
+          const int c = sk[i + u];
+          if (c != cur) {
+            if (cur >= 0) flush(cur);
+            cur = c;
+          }
+          const float s = (sw[i + u] >> 31) ? -1.f : 1.f;
+#pragma unroll
+          for (int j = 0; j < NV; ++j)
+            if ((t + T * j) * EPV < ne) head_add<DT, EPV>(r[u][j], s, acc[j]);
+        }
+    }
+  }
+  if (cur >= 0) flush(cur);
+}
+
+// Y_0 and Y_1 (column-major, J x n) from the row-major J x p accumulators, 32 x 32 tiles; the
+// accumulators are left zero for the next head pass
+__global__ void __launch_bounds__(256) k_head_out(float* __restrict__ Y0r, float* __restrict__ Y1r, float* __restrict__ Y0, float* __restrict__ Y1, int J, int n0,
+                                                   int n1, int p0, int p1, int tiles0) {
+  __shared__ float tl[32][33];
+  const bool first = (int)blockIdx.y < tiles0;
+  float* src = first ? Y0r : Y1r;
+  float* dst = first ? Y0 : Y1;
+  const int n = first ? n0 : n1, p = first ? p0 : p1;
+  const int i0 = 32 * ((int)blockIdx.y - (first ? 0 : tiles0)), b0 = 32 * blockIdx.x;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+  for (int r = y; r < 32; r += 8)
+    if (b0 + r < J && i0 + x < n) {
+      float* q = src + (int64_t)(b0 + r) * p + i0 + x;
+      tl[r][x] = *q;
+      *q = 0.f;
+    }
+  __syncthreads();
+#pragma unroll
+  for (int r = y; r < 32; r += 8)
+    if (b0 + x < J && i0 + r < n) dst[(int64_t)(i0 + r) * J + b0 + x] = tl[x][r];
+}
+
+// ---------------------------------------------------------------------------------------------
+// tail pass
+
+// The plans of both passes for one draw, one CTA each.
+// CTA b < nchunk: the head's pattern of the tail pass, the same for every slab. The entries of a
+// slab, cut into chunks of `chunk` entries, are listed by bucket (sum of the head modes' hashes mod
+// J) within each chunk, in blocks of four 16-bit entry numbers; a bucket's last block is filled up
+// with number `chunk`, an entry that is staged as zero. Bucket word: first block | blocks << 16.
+// Sign word: the signs (product of the head modes' v) of 32 entries.
+// CTA nchunk (when R > 0): the slabs of the head pass sorted by c, the hash of the modes 2 .. d-1
+// (plan word: fibre index of the slab | sign << 31). One CTA sorts up to 2^15 slabs; with more the
+// grid-wide plan of mode 1 (tt_context.cu) is used.
+// Both are counting sorts: counts in shared memory, a scan over the J buckets, placement.
+struct PassPlanArgs {
+  const int32_t* h;
+  const int8_t* v;
+  int64_t n[TT_MAX_D], noff[TT_MAX_D];
+  int d, nh, J, chunk, nchunk, blocks;
+  int64_t E;
+  uint16_t* list;    // 4 * blocks numbers per chunk
+  uint32_t* bucket;  // J words per chunk
+  uint32_t* sign;    // (chunk + 31) / 32 words per chunk
+  int64_t R;         // slabs of the head pass (0: not planned here)
+  uint32_t* plan;
+  int32_t* key;
+};
+constexpr int64_t HEAD_PLAN_MAX = 1 << 15;
+
+__global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
+  extern __shared__ int psm[];  // J counts, then cursors
+  __shared__ int wsum[32];
+  const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5;
+  const bool slabs = (int)blockIdx.x == a.nchunk;
+  const int m0 = slabs ? 2 : 0, m1 = slabs ? a.d : a.nh;  // modes that are hashed
+  const int64_t e0 = slabs ? 0 : (int64_t)blockIdx.x * a.chunk;
+  const int ne = slabs ? (int)a.R : (int)min((int64_t)a.chunk, a.E - e0);
+  for (int b = t; b < a.J; b += T) psm[b] = 0;
+  __syncthreads();
+  auto decode = [&](int i, int& neg) {
+    uint32_t rem = (uint32_t)(e0 + i);
+    int b = 0;
+    neg = 0;
+    for (int s = m0; s < m1; ++s) {
+      const uint32_t n = (uint32_t)a.n[s], q = rem / n, x = rem - q * n;
+      rem = q;
+      b = tt_modj(b + __ldg(a.h + a.noff[s] + x), a.J);
+      neg ^= __ldg(a.v + a.noff[s] + x) < 0;
+    }
+    return b;
+  };
+  uint32_t* sign = a.sign + (int64_t)blockIdx.x * ((a.chunk + 31) / 32);
+  for (int i0 = 0; i0 < ne; i0 += T) {
+    const int i = i0 + t;
+    int neg = 0;
+    if (i < ne) atomicAdd(psm + decode(i, neg), 1);
+    const uint32_t w = __ballot_sync(0xffffffffu, neg);
+    if (!slabs && lane == 0 && i < ne) sign[i >> 5] = w;
+  }
+  __syncthreads();
+  // exclusive scan of the J counts (block counts for a pattern): each thread a run of buckets
+  const int per = (a.J + T - 1) / T, lo = min(a.J, t * per), hi = min(a.J, lo + per);
+  int sum = 0;
+  for (int b = lo; b < hi; ++b) sum += slabs ? psm[b] : (psm[b] + 3) >> 2;
+  int inc = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) wsum[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    int x = wsum[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    wsum[lane] = x;
+  }
+  __syncthreads();
+  int at = (warp ? wsum[warp - 1] : 0) + inc - sum;
+  uint32_t* bucket = a.bucket + (int64_t)blockIdx.x * a.J;
+  uint16_t* list = a.list + (int64_t)blockIdx.x * a.blocks * 4;
+  for (int b = lo; b < hi; ++b) {
+    const int cnt = psm[b];
+    if (slabs) {
+      psm[b] = at;
+      at += cnt;
+    } else {
+      const int nb = (cnt + 3) >> 2;
+      bucket[b] = (uint32_t)at | (uint32_t)nb << 16;
+      for (int i = cnt; i < 4 * nb; ++i) list[4 * at + i] = (uint16_t)a.chunk;
+      psm[b] = 4 * at;
+      at += nb;
+    }
+  }
+  __syncthreads();
+  for (int i = t; i < ne; i += T) {
+    int neg;
+    const int key = decode(i, neg), pos = atomicAdd(psm + key, 1);
+    if (slabs) {
+      a.plan[pos] = (uint32_t)((int64_t)i * a.n[1]) | (uint32_t)neg << 31;
+      a.key[pos] = key;
+    } else {
+      list[pos] = (uint16_t)i;
+    }
+  }
+}
+
+struct TailArgs {
+  const char* A;
+  const float* scales;
+  const uint16_t* list;
+  const uint32_t *bucket, *sign;
+  const int32_t *hs, *hl;  // hashes and signs of the tail modes s (null: one tail mode) and l
+  const int8_t *vs, *vl;
+  float *Ys, *Yl;  // J x n_s, J x n_l column-major, zeroed
+  int64_t E;       // entries of a slab
+  int J, n0, chunk, nchunk, blocks, ns, nl, ngl;  // ngl: groups of V indices i_l
+  int parts;       // lanes that share a bucket's list (a power of two)
+  uint32_t inv_n0;  // 2^32 / n_0 rounded up (FP8: entry number -> i_0)
+  int64_t units;   // nchunk * ngl * ns
+};
+
+constexpr int TAIL_T = 1024;
+
+// What a thread stages per slab group: JJ loads of EPW entries from each of V slabs. An entry of the
+// staged chunk holds its V slabs' signed values side by side (V * SB bytes), so that one
+// shared-memory load per list number serves V slabs. FP64 is staged as FP32.
+template <int DT, int V, int EPW>
+struct TailShape {
+  static constexpr int EB = TtElem<DT>::bytes;
+  static constexpr int SB = EB == 8 ? 4 : EB;
+  static constexpr int JJ = EB == 8 ? 5 : 20 / V;
+  static constexpr int ENT = V * SB;  // bytes of a staged entry
+};
+
+// x + y in one instruction
+__device__ __forceinline__ float2 add2(float2 x, float2 y) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y));
+  return d;
+}
+
+// One CTA of 1024 threads per SM; unit = (chunk, group of V indices i_l, i_s), consecutive units in one
+// CTA. Thread t owns bucket b of Y_l and so, per i_s, the head's bucket b - h_s(i_s): it sums that
+// bucket's list from the staged slabs (random 8-byte shared-memory loads), keeps Y_l's column sums in
+// registers while i_s advances, and adds its q to Y_s with atomics that are contiguous across a warp.
+// The next unit's slabs are loaded into registers meanwhile. The signs go on when a slab is staged.
+// Bound: instruction issue (61% active; 115 M warp instructions) and the random shared-memory loads
+// (150 k of 331 k cycles). 100^4 FP32: 160 us for both modes at J = 4096, 134 us at J = 1024 (one
+// launch per mode: 206 and 172 us).
+template <int DT, int V, int EPW, int RPT>
+__global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
+  using Sh = TailShape<DT, V, EPW>;
+  constexpr int EB = Sh::EB, JJ = Sh::JJ, ENT = Sh::ENT, T = TAIL_T;
+  using Word = typename std::conditional<EB == 8, double, uint32_t>::type;
+  extern __shared__ __align__(16) unsigned char tsm[];
+  unsigned char* buf = tsm;                                                                  // chunk + 1 entries
+  uint2* sl = reinterpret_cast<uint2*>(buf + (((size_t)(a.chunk + 1) * ENT + 15) & ~(size_t)15));  // blocks
+  uint32_t* sb = reinterpret_cast<uint32_t*>(sl + a.blocks);                                 // J
+  float* ssc = reinterpret_cast<float*>(sb + a.J);                                           // n0 FP8 scales
+  const int t = threadIdx.x, J = a.J, parts = a.parts;
+  const int part = t & (parts - 1), row0 = t / parts, rstep = T / parts;
+  if (DT == TT_FP8E4M3)
+    for (int i = t; i < a.n0; i += T) ssc[i] = __ldg(a.scales + i);
+  if (t < ENT) buf[(size_t)a.chunk * ENT + t] = 0;
+  const int64_t u0 = a.units * blockIdx.x / gridDim.x, u1 = a.units * (blockIdx.x + 1) / gridDim.x;
+  if (u0 >= u1) return;
+  int is = (int)(u0 % a.ns), gl = (int)((u0 / a.ns) % a.ngl), ch = (int)(u0 / a.ns / a.ngl);
+
+  Word pw[JJ][V];
+  int nj = 0;  // loads of this thread in the chunk last fetched
+  // slabs past the last index l read the last one's values, which are not added to any column
+  auto fetch = [&](int ch_, int gl_, int is_) {
+    const int ne = (int)min((int64_t)a.chunk, a.E - (int64_t)ch_ * a.chunk);
+    nj = (ne / EPW - t + T - 1) / T;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const int il = min(V * gl_ + v, a.nl - 1);
+      const char* p = a.A + (((int64_t)il * a.ns + is_) * a.E + (int64_t)ch_ * a.chunk) * EB + t * (EPW * EB);
+#pragma unroll
+      for (int jj = 0; jj < JJ; ++jj) {
+        if (jj < nj) {
+          const char* q = p + T * jj * (EPW * EB);
+          if constexpr (EPW * EB == 8) pw[jj][v] = __ldg(reinterpret_cast<const double*>(q));
+          else if constexpr (EPW * EB == 4) pw[jj][v] = __ldg(reinterpret_cast<const uint32_t*>(q));
+          else if constexpr (EPW * EB == 2) pw[jj][v] = __ldg(reinterpret_cast<const unsigned short*>(q));
+          else pw[jj][v] = __ldg(reinterpret_cast<const unsigned char*>(q));
+        }
+      }
+    }
+  };
+  uint32_t smask = 0;  // signs of this thread's entries, bit EPW * jj + e
+  auto stage = [&]() {
+#pragma unroll
+    for (int jj = 0; jj < JJ; ++jj) {
+      if (jj >= nj) continue;
+      unsigned char* dst = buf + (size_t)((t + T * jj) * EPW) * ENT;
+      if constexpr (EB == 8) {
+        const float s = __uint_as_float(0x3F800000u | (smask << (31 - jj) & 0x80000000u));
+        *reinterpret_cast<float2*>(dst) = make_float2(s * (float)pw[jj][0], s * (float)pw[jj][1]);
+      } else if constexpr (EB == 4) {
+        const uint32_t m = smask << (31 - jj) & 0x80000000u;
+        *reinterpret_cast<uint2*>(dst) = make_uint2(pw[jj][0] ^ m, pw[jj][1] ^ m);
+      } else if constexpr (EB == 2 && EPW == 2) {
+        const uint32_t m = (smask >> (2 * jj) & 1u) << 15 | (smask >> (2 * jj + 1) & 1u) << 31;
+        uint32_t w[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) w[v] = pw[jj][v] ^ m;
+        *reinterpret_cast<uint4*>(dst) = make_uint4(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410),
+                                                    __byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632));
+      } else if constexpr (EB == 2) {
+        const uint32_t m = (smask >> jj & 1u) * 0x80008000u;
+        *reinterpret_cast<uint32_t*>(dst) = (pw[jj][0] | pw[jj][1] << 16) ^ m;
+      } else if constexpr (EPW == 4) {
+        const uint32_t m = ((smask >> (4 * jj) & 15u) * 0x00204081u & 0x01010101u) << 7;
+        uint32_t w[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) w[v] = pw[jj][v] ^ m;
+        const uint32_t t0 = __byte_perm(w[0], w[1], 0x5140), t1 = __byte_perm(w[2], w[3], 0x5140);
+        const uint32_t t2 = __byte_perm(w[0], w[1], 0x7362), t3 = __byte_perm(w[2], w[3], 0x7362);
+        *reinterpret_cast<uint4*>(dst) = make_uint4(__byte_perm(t0, t1, 0x5410), __byte_perm(t0, t1, 0x7632),
+                                                    __byte_perm(t2, t3, 0x5410), __byte_perm(t2, t3, 0x7632));
+      } else {
+        *reinterpret_cast<unsigned short*>(dst) =
+            (unsigned short)((pw[jj][0] | pw[jj][1] << 8) ^ (smask >> jj & 1u) * 0x8080u);
+      }
+    }
+  };
+  int i0base = 0;  // i_0 of the chunk's first entry
+  // q += the V values of the chunk's entry number x
+  auto gather = [&](uint32_t x, float (&q)[V]) {
+    const unsigned char* src = buf + x * ENT;
+    if constexpr (EB >= 4) {
+      const float2 r = add2(make_float2(q[0], q[1]), *reinterpret_cast<const float2*>(src));
+      q[0] = r.x, q[1] = r.y;
+    } else if constexpr (EB == 2) {
+      tt_fma_bf16x2(*reinterpret_cast<const uint32_t*>(src), 0x3F80, q[0], q[1]);
+      if constexpr (V == 4) tt_fma_bf16x2(*reinterpret_cast<const uint32_t*>(src + 4), 0x3F80, q[2], q[3]);
+    } else {
+      const uint32_t y = x + i0base;
+      const float s = ssc[y - __umulhi(y, a.inv_n0) * a.n0];
+      if constexpr (V == 4) {
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        tt_fma_e4m3x4(*reinterpret_cast<const uint32_t*>(src), 0x3C00, d[0], d[1], d[2], d[3]);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) q[v] = fmaf(s, d[v], q[v]);
+      } else {
+        const uint32_t w = *reinterpret_cast<const unsigned short*>(src);
+        q[0] = fmaf(s, tt_e4m3_to_float(w), q[0]);
+        q[1] = fmaf(s, tt_e4m3_to_float(w >> 8), q[1]);
+      }
+    }
+  };
+  float acc[RPT][V];
+#pragma unroll
+  for (int j = 0; j < RPT; ++j)
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[j][v] = 0.f;
+  auto flush = [&](int gl_) {  // the group's columns of Y_l
+    if (part == 0) {
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        const int b = row0 + rstep * j;
+        if (b < J) {
+#pragma unroll
+          for (int v = 0; v < V; ++v)
+            if (V * gl_ + v < a.nl && acc[j][v] != 0.f) atomicAdd(a.Yl + (int64_t)J * (V * gl_ + v) + b, acc[j][v]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < RPT; ++j)
+#pragma unroll
+      for (int v = 0; v < V; ++v) acc[j][v] = 0.f;
+  };
+
+  fetch(ch, gl, is);
+  int ch_in = -1;
+  for (int64_t u = u0; u < u1; ++u) {
+    __syncthreads();  // the staged chunk and lists are no longer read
+    if (ch != ch_in) {
+      const uint2* gl2 = reinterpret_cast<const uint2*>(a.list) + (int64_t)ch * a.blocks;
+      for (int i = t; i < a.blocks; i += T) sl[i] = __ldg(gl2 + i);
+      for (int b = t; b < J; b += T) sb[b] = __ldg(a.bucket + (int64_t)ch * J + b);
+      const uint32_t* sg = a.sign + (int64_t)ch * ((a.chunk + 31) / 32);
+      smask = 0;
+#pragma unroll
+      for (int jj = 0; jj < JJ; ++jj) {
+        const int i = (t + T * jj) * EPW;
+        if (jj < nj) smask |= (__ldg(sg + (i >> 5)) >> (i & 31) & ((1u << EPW) - 1u)) << (EPW * jj);
+      }
+      if (DT == TT_FP8E4M3) i0base = (int)((int64_t)ch * a.chunk % a.n0);
+      ch_in = ch;
+    }
+    stage();
+    __syncthreads();
+    int nis = is + 1, ngl = gl, nch = ch;
+    if (nis == a.ns) {
+      nis = 0;
+      if (++ngl == a.ngl) ngl = 0, ++nch;
+    }
+    if (u + 1 < u1) fetch(nch, ngl, nis);  // in flight during the sums below
+    int hs = 0;
+    float vs = 1.f;
+    int hl[V];
+    float vl[V];
+    float* ys = nullptr;
+    const int nv = min(V, a.nl - V * gl);
+    if (a.hs) {
+      hs = __ldg(a.hs + is);
+      vs = __ldg(a.vs + is) < 0 ? -1.f : 1.f;
+      ys = a.Ys + (int64_t)J * is;
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int il = min(V * gl + v, a.nl - 1);
+        hl[v] = __ldg(a.hl + il);
+        vl[v] = __ldg(a.vl + il) < 0 ? -1.f : 1.f;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+      const int b = row0 + rstep * j;  // bucket of Y_l; the head's bucket c = b - h_s(i_s)
+      if (RPT > 1 && rstep * j >= J) break;
+      int c = b - hs;
+      if (c < 0) c += J;
+      const uint32_t se = b < J ? sb[c] : 0u;
+      const int p0 = (int)(se & 0xFFFFu), pe = p0 + (int)(se >> 16);
+      float q[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) q[v] = 0.f;
+      for (int p = p0 + part; p < pe; p += parts) {
+        const uint2 x = sl[p];
+        gather(x.x & 0xFFFFu, q);
+        gather(x.x >> 16, q);
+        gather(x.y & 0xFFFFu, q);
+        gather(x.y >> 16, q);
+      }
+      if (parts > 1)
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          for (int o = 1; o < parts; o <<= 1) q[v] += __shfl_xor_sync(0xffffffffu, q[v], o);
+#pragma unroll
+      for (int v = 0; v < V; ++v) acc[j][v] = fmaf(vs, q[v], acc[j][v]);
+      if (a.hs && part == 0 && pe > p0) {
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          if (v < nv) atomicAdd(ys + tt_modj(c + hl[v], J), vl[v] * q[v]);
+      }
+    }
+    if (ngl != gl || nch != ch || u + 1 == u1) flush(gl);
+    is = nis, gl = ngl, ch = nch;
+  }
+}
+
+// CTAs of a pass with per_sm resident on an SM: one wave.
+// - Beside the chain of a single-tensor sweep it covers four fifths of the SMs: the passes' CTAs hold
+//   an SM's registers until they end, and the chain's kernels run on the others (100^4 FP32: 732 us
+//   per monitored sweep with a whole wave, 674, 639 and 640 us with 136, 120 and 104 tail CTAs, 626
+//   with the head pass cut the same way).
+// - In a batch at most one CTA per half an item's bytes, so that small tensors' passes run side by
+//   side (256 tensors: 14.50 ms per batched sweep without the bound, 13.83 ms with it; 32 tensors:
+//   2.50 ms; 2.81, 2.41, 2.40 and 2.46 ms at 1 MB, 512, 256 and 128 KB per CTA).
+int64_t pass_ctas(const tt_ctx* c, int per_sm) {
+  const int64_t sms = tt_sm_count();
+  const int64_t covered = c->in_sweep && !c->capture_mode ? sms * 4 / 5 : sms;
+  int64_t ctas = std::max<int64_t>(1, covered) * std::max(1, per_sm);
+  if (c->item_bytes > 0) ctas = std::min(ctas, 2 * c->N * tt_elem_bytes(c->dtype) / c->item_bytes);
+  return std::max<int64_t>(1, ctas);
+}
+
+template <int DT, int V, int EPW>
+int launch_tail_v(tt_ctx* c, TailArgs a) {
+  using Sh = TailShape<DT, V, EPW>;
+  a.ngl = (a.nl + V - 1) / V;
+  a.units = (int64_t)a.nchunk * a.ngl * a.ns;
+  a.parts = 1;
+  while (a.parts < 8 && 2 * a.parts * a.J <= TAIL_T) a.parts *= 2;
+  const size_t smem = (((size_t)(a.chunk + 1) * Sh::ENT + 15) & ~(size_t)15) + 8 * (size_t)a.blocks + 4 * (size_t)a.J +
+                      (DT == TT_FP8E4M3 ? 4 * (size_t)a.n0 : 0);
+  void (*kern)(TailArgs) = a.J <= 1024   ? k_tail_pass<DT, V, EPW, 1>
+                           : a.J <= 2048 ? k_tail_pass<DT, V, EPW, 2>
+                           : a.J <= 4096 ? k_tail_pass<DT, V, EPW, 4>
+                                         : k_tail_pass<DT, V, EPW, 8>;
+  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int blocks = (int)std::min<int64_t>(a.units, pass_ctas(c, 1));
+  kern<<<blocks, TAIL_T, smem, c->stream>>>(a);
+  TT_LAUNCH(c, "k_tail_pass");
+  return TT_OK;
+}
+
+template <int DT>
+int launch_tail(tt_ctx* c, const TailArgs& a) {
+  constexpr int EB = TtElem<DT>::bytes;
+  if constexpr (EB >= 4) {
+    return launch_tail_v<DT, 2, 1>(c, a);
+  } else {
+    // 32-bit loads where every slab starts on a 4-byte boundary
+    if (reinterpret_cast<uintptr_t>(a.A) % 4 == 0 && a.E * EB % 4 == 0) return launch_tail_v<DT, 4, 4 / EB>(c, a);
+    return launch_tail_v<DT, 2, 1>(c, a);
+  }
+}
+
+template <int DT, int VB>
+int launch_head_vb(tt_ctx* c, HeadArgs a) {
+  constexpr int PT = 32 * head_acc<DT>();  // entries per warp
+  const int threads = (int)(((int64_t)a.n0 * a.G1 + PT - 1) / PT) * 32;
+  const int rows = (a.G1 + 3) & ~3;
+  const size_t smem = sizeof(float) * ((size_t)rows * a.pitch + 3 * (size_t)((a.n0 + 3) & ~3) + rows + 2 * HEAD_BATCH);
+  auto kern = k_head_pass<DT, VB>;
+  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 1;
+  TT_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+  a.nseg = (int)std::max<int64_t>(1, std::min<int64_t>(a.R, pass_ctas(c, per_sm) / a.nch));
+  kern<<<a.nseg * a.nch, threads, smem, c->stream>>>(a);
+  TT_LAUNCH(c, "k_head_pass");
+  return TT_OK;
+}
+
+// the widest vectors that slabs and chunks start on (a column need not)
+template <int DT>
+int launch_head(tt_ctx* c, const HeadArgs& a) {
+  constexpr int EB = TtElem<DT>::bytes;
+  const uint64_t at = reinterpret_cast<uintptr_t>(a.A) | (uint64_t)a.n0 * a.n1 * EB | (a.nch > 1 ? (uint64_t)a.n0 * a.G1 * EB : 0);
+  if (at % 16 == 0) return launch_head_vb<DT, 16>(c, a);
+  if (at % 8 == 0) return launch_head_vb<DT, 8>(c, a);
+  if constexpr (EB <= 4)
+    if (at % 4 == 0) return launch_head_vb<DT, 4>(c, a);
+  if constexpr (EB < 4) return launch_head_vb<DT, EB>(c, a);
+  return tt_fail(c, TT_EINVAL, "A is not aligned to its storage type");
+}
+
+int head_cols(const tt_ctx* c) {  // columns i_1 per chunk
+  // at most what the threads hold, and 128 KB of transposition tile
+  const int64_t cap = std::min<int64_t>(HEAD_TMAX * (c->dtype == TT_F64 ? head_acc<TT_F64>() : head_acc<TT_F32>()) / c->n[0],
+                                        (128 * 1024 / 4) / ((c->n[0] + 31) & ~31));
+  if (cap >= c->n[1]) return (int)c->n[1];
+  const int64_t nch = (c->n[1] + (cap & ~3) - 1) / std::max<int64_t>(4, cap & ~3);
+  return (int)(((c->n[1] + nch - 1) / nch + 3) & ~3);
+}
+
+// entries per chunk: what a CTA's threads can fetch at once (JJ loads each; the narrow loads' reach)
+int64_t tail_chunk_max(const tt_ctx* c) { return c->dtype == TT_F64 ? TAIL_T * 5 : TAIL_T * 10; }
+
+}  // namespace
+
+// Which modes the passes cover, from the shape alone. Workspaces of both sketch draws follow from it.
+// The head pass needs slabs that fill a CTA's warps (512 entries) and columns that leave room for four
+// in a chunk; its row accumulators stay in L2 (32 MB). The tail pass needs chunks of at least that
+// size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. J up to 8192:
+// eight buckets per thread. The deterministic mode has its own kernels; the batch autotuner times
+// launches per mode.
+void tt_pass_plan(tt_ctx* c) {
+  c->pass_head = c->pass_tail = false;
+  c->tail_modes = 0;
+  if (c->det || (c->flags & TT_FLAG_BATCH_AUTOTUNE) || c->J > 8192) return;
+  const int64_t e2 = c->n[0] * c->n[1];
+  c->p0 = (int)((c->n[0] + 3) & ~3);
+  c->p1 = (int)((c->n[1] + 3) & ~3);
+  c->pass_head = e2 >= 512 && c->n[0] <= HEAD_TMAX * head_acc<TT_F64>() / 4 && (int64_t)c->J * (c->p0 + c->p1) <= (8 << 20);
+  const int nt = c->d >= 4 ? 2 : c->d == 3 ? 1 : 0;
+  if (nt) {
+    const int64_t E = c->stride[c->d - nt];
+    const int64_t cm = tail_chunk_max(c);
+    c->tail_nchunk = (int)((E + cm - 1) / cm);
+    c->tail_chunk = (int)(((E + c->tail_nchunk - 1) / c->tail_nchunk + 3) & ~3);
+    // a bucket's blocks: all full but its last one
+    c->tail_blocks = c->tail_chunk / 4 + std::min(c->J, c->tail_chunk);
+    c->pass_tail = E >= 512 && E * 8 >= c->J && c->tail_nchunk <= 64;
+    if (c->pass_tail) c->tail_modes = nt;
+  }
+  c->head_sorted = c->pass_head && c->N / e2 <= HEAD_PLAN_MAX;
+}
+
+unsigned tt_pass_mask(const tt_ctx* c) {
+  unsigned m = c->pass_head ? 3u : 0u;
+  for (int s = 0; s < c->tail_modes; ++s) m |= 1u << (c->d - 1 - s);
+  return m;
+}
+
+// modes whose fibre plan an all-modes data sketch reads: every mode without a pass, and mode 1 where
+// the head pass takes its slabs from it
+unsigned tt_pass_plans(const tt_ctx* c) {
+  return (((1u << c->d) - 1u) & ~tt_pass_mask(c)) | (c->pass_head && !c->head_sorted ? 2u : 0u);
+}
+
+int tt_launch_pass_plans(tt_ctx* c) {
+  PassPlanArgs p{};
+  p.h = c->d_h;
+  p.v = c->d_v;
+  p.d = c->d;
+  p.nh = c->d - c->tail_modes;
+  for (int s = 0; s < TT_MAX_D; ++s) {
+    p.n[s] = s < c->d ? c->n[s] : 1;
+    p.noff[s] = s < c->d ? c->noff[s] : 0;
+  }
+  p.J = c->J;
+  p.chunk = c->tail_chunk;
+  p.nchunk = c->pass_tail ? c->tail_nchunk : 0;
+  p.blocks = c->tail_blocks;
+  p.E = c->stride[p.nh];
+  p.list = c->d_tlist;
+  p.bucket = c->d_tbucket;
+  p.sign = c->d_tbucket + (int64_t)c->J * c->tail_nchunk;
+  p.R = c->head_sorted ? c->R[1] : 0;
+  p.plan = c->d_hplan;
+  p.key = c->d_rkey;
+  const int ctas = p.nchunk + (c->head_sorted ? 1 : 0);
+  if (ctas == 0) return TT_OK;
+  k_pass_plans<<<ctas, 1024, sizeof(int) * (size_t)c->J, c->stream>>>(p);
+  TT_LAUNCH(c, "k_pass_plans");
+  return TT_OK;
+}
+
+int tt_launch_head_pass(tt_ctx* c, const void* A, const float* scales, float* const* Y) {
+  HeadArgs a{};
+  a.A = (const char*)A;
+  a.scales = scales;
+  a.plan = c->head_sorted ? c->d_hplan : c->d_rplan[1];
+  a.key = c->d_rkey;
+  a.h0 = c->d_h;
+  a.v0 = c->d_v;
+  a.h1 = c->d_h + c->noff[1];
+  a.v1 = c->d_v + c->noff[1];
+  a.R = c->R[1];
+  a.J = c->J;
+  a.n0 = (int)c->n[0];
+  a.n1 = (int)c->n[1];
+  a.p0 = c->p0;
+  a.p1 = c->p1;
+  a.Y0r = c->d_y01;
+  a.Y1r = c->d_y01 + (int64_t)c->J * c->p0;
+  a.G1 = head_cols(c);
+  a.nch = (a.n1 + a.G1 - 1) / a.G1;
+  a.pitch = (a.n0 + 31) & ~31;
+  a.inv_n0 = (uint32_t)((((uint64_t)1 << 32) + a.n0 - 1) / a.n0);
+  for (int z = 0; z < c->tail_modes; ++z) {
+    a.zero[z] = Y[c->d - 1 - z];
+    a.nzero[z] = (int64_t)c->J * c->n[c->d - 1 - z];
+  }
+  if (!c->y01_zero) TT_CUDA(c, cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)c->J * (c->p0 + c->p1), c->stream));
+  c->y01_zero = false;
+  switch (c->dtype) {
+    case TT_F64: TT_TRY(launch_head<TT_F64>(c, a)); break;
+    case TT_F32: TT_TRY(launch_head<TT_F32>(c, a)); break;
+    case TT_BF16: TT_TRY(launch_head<TT_BF16>(c, a)); break;
+    default: TT_TRY(launch_head<TT_FP8E4M3>(c, a)); break;
+  }
+  const int t0 = (a.n0 + 31) / 32, t1 = (a.n1 + 31) / 32;
+  k_head_out<<<dim3((c->J + 31) / 32, t0 + t1), 256, 0, c->stream>>>(a.Y0r, a.Y1r, Y[0], Y[1], c->J, a.n0, a.n1, a.p0, a.p1, t0);
+  TT_LAUNCH(c, "k_head_out");
+  c->y01_zero = true;
+  return TT_OK;
+}
+
+int tt_launch_tail_pass(tt_ctx* c, const void* A, const float* scales, float* Ys, float* Yl) {
+  const int l = c->d - 1, s = c->d - 2;
+  TailArgs a{};
+  a.A = (const char*)A;
+  a.scales = scales;
+  a.list = c->d_tlist;
+  a.bucket = c->d_tbucket;
+  a.sign = c->d_tbucket + (int64_t)c->J * c->tail_nchunk;
+  a.blocks = c->tail_blocks;
+  a.inv_n0 = (uint32_t)((((uint64_t)1 << 32) + c->n[0] - 1) / c->n[0]);
+  a.hl = c->d_h + c->noff[l];
+  a.vl = c->d_v + c->noff[l];
+  if (c->tail_modes == 2) {
+    a.hs = c->d_h + c->noff[s];
+    a.vs = c->d_v + c->noff[s];
+    a.Ys = Ys;
+  }
+  a.Yl = Yl;
+  for (int k = l; k > l - c->tail_modes && !c->pass_head; --k)  // (the head pass zeroes them)
+    TT_CUDA(c, cudaMemsetAsync(k == l ? Yl : Ys, 0, sizeof(float) * (size_t)c->J * c->n[k], c->stream));
+  a.E = c->stride[c->d - c->tail_modes];
+  a.J = c->J;
+  a.n0 = (int)c->n[0];
+  a.chunk = c->tail_chunk;
+  a.nchunk = c->tail_nchunk;
+  a.ns = c->tail_modes == 2 ? (int)c->n[s] : 1;
+  a.nl = (int)c->n[l];
+  switch (c->dtype) {
+    case TT_F64: return launch_tail<TT_F64>(c, a);
+    case TT_F32: return launch_tail<TT_F32>(c, a);
+    case TT_BF16: return launch_tail<TT_BF16>(c, a);
+    default: return launch_tail<TT_FP8E4M3>(c, a);
+  }
+}
+
+// The data sketches of all modes on c->stream: the passes, then one launch per remaining mode; ev[k]
+// (when given) is recorded after Y_k.
+int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev) {
+  TT_TRY(tt_ensure_plans(c, tt_pass_plans(c), true));
+  const unsigned mask = tt_pass_mask(c);
+  const int64_t bytes = c->N * tt_elem_bytes(c->dtype) + (c->dtype == TT_FP8E4M3 ? 4 * c->n[0] : 0);
+  auto mark = [&](int k) -> int {  // Y_k is done
+    if (ev) TT_CUDA(c, cudaEventRecord(ev[k], c->stream));
+    return TT_OK;
+  };
+  // a pass is timed as its first mode, its other modes as empty intervals (its bytes count once)
+  auto timed = [&](int k0, int k1, auto&& pass) -> int {
+    TT_TRY(tt_prof_begin(c, k0));
+    TT_TRY(pass());
+    TT_TRY(tt_prof_end(c));
+    for (int k = k0 + 1; k <= k1; ++k) {
+      TT_TRY(tt_prof_begin(c, k));
+      TT_TRY(tt_prof_end(c));
+      if (c->profiling) c->prof_bytes -= bytes;
+    }
+    for (int k = k0; k <= k1; ++k) TT_TRY(mark(k));
+    return TT_OK;
+  };
+  if (c->pass_head) TT_TRY(timed(0, 1, [&] { return tt_launch_head_pass(c, A, scales, Y); }));
+  for (int k = 0; k < c->d; ++k)
+    if (!(mask & (1u << k))) {
+      TT_TRY(tt_launch_unfold_planned(c, A, scales, k, Y[k]));
+      TT_TRY(mark(k));
+    }
+  const int l = c->d - 1;
+  if (c->pass_tail)
+    TT_TRY(timed(c->d - c->tail_modes, l, [&] { return tt_launch_tail_pass(c, A, scales, Y[l - 1], Y[l]); }));
+  return TT_OK;
+}

@@ -325,9 +325,12 @@ int tt_launch_unfold(tt_ctx* c, const void* A, const float* scales, int k, float
     ys[k] = Y;
     return tt_launch_unfold_det(c, A, scales, 1u << k, ys);
   }
-  int rc = tt_ensure_rplan(c, k);  // plan build is not part of the timed kernel
-  if (rc) return rc;
-  rc = tt_prof_begin(c, k);
+  TT_TRY(tt_ensure_rplan(c, k));  // plan build is not part of the timed kernel
+  return tt_launch_unfold_planned(c, A, scales, k, Y);
+}
+
+int tt_launch_unfold_planned(tt_ctx* c, const void* A, const float* scales, int k, float* Y) {
+  int rc = tt_prof_begin(c, k);
   if (rc) return rc;
   switch (c->dtype) {
     case TT_F64: rc = unfold_dt<TT_F64>(c, A, scales, k, Y); break;

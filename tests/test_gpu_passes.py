@@ -1,0 +1,102 @@
+"""Data sketches of all modes from passes over A that serve two modes each (Alg. 1 part (a)): modes 0
+and 1 from one read, the last one or two modes from another. Every mode against the oracle's sketch by
+definition, in every storage type, at the edges of the passes' tiles: slabs of one and of several
+chunks (10,240 entries; 5,120 in FP64), chunks that end inside a column, slabs on 16-, 8-, 4-, 2- and
+1-byte boundaries, odd groups of tail indices, sketch sizes from fewer buckets than a CTA's threads
+share up to 8192, more slabs than one CTA sorts, and tensors that start off the 16-byte grid. The
+tolerance is the suite's for FP32 sums (1e-5 relative)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+import tt_oracle as O  # noqa: E402
+from paper_2309_08093_gb300 import lib, synth  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+SHAPES = [  # dims, J
+    ((50, 50, 50), 1024),
+    ((24, 23), 64),               # order 2: the head pass alone
+    ((33, 31, 17), 512),          # odd columns
+    ((101, 84, 9, 5), 128),       # eight lanes per bucket list
+    ((128, 80, 3, 5), 2048),      # a slab of exactly 10,240 entries
+    ((128, 81, 3, 5), 2047),      # one column more: two chunks; J not a power of two
+    ((12, 11, 10, 9, 8), 4096),   # order 5: a mode between the passes
+    ((6, 7, 29, 3, 2, 2), 1200),  # order 6: modes 0 and 1 without a pass
+    ((30, 30, 14, 7, 3), 8192),   # several chunks, the largest J
+    ((2048, 5, 6), 512),          # columns that leave four to a chunk
+    ((8, 300, 5, 4), 45),
+]
+
+
+def _check(dims, J, dtype, offset=0, columns=None):
+    seed = 977
+    a = synth.random_tensor(dims, 31)
+    flat, scales, exact = synth.quantize(a, dtype)
+    A = lib.device_tensor(np.concatenate([np.zeros(offset, flat.dtype), flat]), dtype)[offset:]
+    sc = torch.from_numpy(scales).cuda() if scales is not None else None
+    ctx = lib.Context(dims, [1] + [2] * (len(dims) - 1) + [1], J, 1e-3, seed, dtype)
+    Y = [torch.full((n, J), 3.0, device="cuda") for n in dims]
+    for sweep in (4, 5):  # a second draw: accumulators and plans of the first are gone
+        ctx.tt_sketch_unfold(A, -1, sweep, Y, sc)
+    hs, vs = O.draw_sketch(seed, 5, dims, J)
+    for k, n in enumerate(dims):
+        cols = range(n) if columns is None else sorted({0, n // 2, n - 1})
+        ref = np.stack([O.sketch_unfolding_column(exact, hs, vs, J, k, i) for i in cols])
+        got = Y[k][list(cols)].double().cpu().numpy()
+        err = np.linalg.norm(got - ref) / np.linalg.norm(ref)
+        assert err <= TOL, (dims, J, dtype, k, err)
+        # a bucket's error against the terms it sums: a lost or mis-signed term shows
+        mag = np.stack([O.sketch_unfolding_column(np.abs(exact), hs, [np.ones_like(v) for v in vs], J, k, i)
+                        for i in cols])
+        assert np.all(np.abs(got - ref) <= TOL * (mag + np.abs(exact).max())), (dims, J, dtype, k)
+    ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16", "fp8"])
+@pytest.mark.parametrize("dims,J", SHAPES)
+def test_all_modes_against_the_oracle(dims, J, dtype):
+    _check(dims, J, dtype)
+
+
+@pytest.mark.parametrize("dtype,offset", [("f32", 1), ("f32", 2), ("f64", 1), ("bf16", 1), ("bf16", 2), ("bf16", 4),
+                                          ("fp8", 1), ("fp8", 2), ("fp8", 4), ("fp8", 8)])
+def test_tensor_off_the_16_byte_grid(dtype, offset):
+    _check((32, 24, 7, 5), 256, dtype, offset)
+
+
+def test_more_slabs_than_one_cta_sorts():
+    """33,800 slabs of 512 entries: the head pass takes them from mode 1's grid-wide plan."""
+    _check((32, 16, 130, 260), 1024, "f32", columns=3)
+
+
+def test_a_workspace_cap_that_leaves_no_room_for_the_passes():
+    """A cap between the needs of one launch per mode and of the passes: the context is created, and
+    its sketches are the same."""
+    dims, J, seed = (40, 36, 10, 9), 1024, 5
+    ranks = (1, 2, 2, 2, 1)
+    A = lib.device_tensor(synth.quantize(synth.random_tensor(dims, 3), "f32")[0], "f32")
+    Y = [[torch.empty(n, J, device="cuda") for n in dims] for _ in range(2)]
+    ctx = lib.Context(dims, ranks, J, 1e-3, seed)
+    ctx.tt_sketch_unfold(A, -1, 0, Y[0])
+    ctx.close()
+    lo, hi = 1 << 16, 1 << 26  # smallest cap that still creates a context
+    prev = lib.tt_set_workspace_limit(0)
+    try:
+        while hi - lo > 4096:
+            mid = (lo + hi) // 2
+            lib.tt_set_workspace_limit(mid)
+            try:
+                lib.Context(dims, ranks, J, 1e-3, seed).close()
+                hi = mid
+            except lib.TtError:
+                lo = mid
+        lib.tt_set_workspace_limit(hi)
+        ctx = lib.Context(dims, ranks, J, 1e-3, seed)
+    finally:
+        lib.tt_set_workspace_limit(prev)
+    ctx.tt_sketch_unfold(A, -1, 0, Y[1])
+    for a, b in zip(*Y):
+        assert float(torch.linalg.vector_norm(a - b)) <= TOL * float(torch.linalg.vector_norm(a))
+    ctx.close()

@@ -346,8 +346,12 @@ int tt_launch_gram_tc(tt_ctx* c, const float* SH, const float* Y, int s, int n, 
 int tt_launch_prox_update64(tt_ctx* c, const float* Y, const float* SH, float* core, int k, double* change_slot,
                             bool gram_zeroed);
 int tt_launch_qr_left(tt_ctx* c, float* core_k, float* core_k1, int k);
-int tt_launch_lq_right(tt_ctx* c, float* core_km1, float* core_k, int k);
+int tt_launch_lq_right(tt_ctx* c, float* const* cores, int k);
 int tt_launch_lq_sweep(tt_ctx* c, float* const* cores);  // all right-to-left steps
+// tt_qr.cu: the QR step of core k / the right-to-left steps k1 .. k0; false (nothing launched) when a
+// rank exceeds 32 or an unfolding its shared memory
+bool tt_qr_left_tiles(tt_ctx* c, float* core, float* next, int k, cudaError_t* err);
+bool tt_lq_tiles(tt_ctx* c, float* const* cores, int k1, int k0, cudaError_t* err);
 int tt_launch_rel_error(tt_ctx* c, const void* A, const float* scales, float* const* cores,
                         double* acc = nullptr);  // acc: 2 doubles (default: the context's)
 int tt_read_status(tt_ctx* c);

@@ -6,10 +6,8 @@
 //                   256 rows and across chunks (split-K, FP32 atomics)
 //   k_prox_solve  : Gauss-Jordan elimination of [M | B^T] in registers, one barrier per pivot,
 //                   one CTA per chunk of right-hand-side rows (s <= 160)
-//   k_qr_left_rows, k_lq_right_rows : CholeskyQR2 with rows in registers (rank <= 16), then
-//                   G_k <- Q and R absorbed into the neighbour (prefetched during the QR)
-//   k_qr_left     : the same for larger ranks (Gram in shared memory), Householder fallback:
-//                   G_k^L = Q R, G_k <- Q, G_{k+1} <- R G_{k+1}^R
+//   k_qr_left     : the QR step of cores beyond the kernels of tt_qr.cu: G_k^L = Q R, G_k <- Q,
+//                   G_{k+1} <- R G_{k+1}^R
 //   k_lq_right    : the same on (G_k^R)^T: G_k^R <- Q^T, G_{k-1}^L <- G_{k-1}^L R^T
 //   k_slab_u, k_rint, k_rel_error_stream : ||A - [[G]]||_F^2 and ||A||_F^2: right interfaces of
 //                   all mode-0 fibres, then one pass over A in memory order (bulk copies)
@@ -19,6 +17,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "tt_householder.cuh"
 #include "tt_internal.cuh"
 
 // 4-byte asynchronous copies global -> shared (cp.async), committed and awaited by group
@@ -584,97 +583,8 @@ int tt_launch_prox_update(tt_ctx* c, const float* Y, const float* SH, float* cor
 }
 
 // ---------------------------------------------------------------------------------------------
-// Householder QR of an m x q column-major matrix held in shared memory (q small).
-// On exit: A holds Q (m x p, p = min(m, q)) in its first p columns, R (p x q) in Rm (q x q,
-// row-major, rows >= p zero), with diag(R) >= 0.
-
-__device__ float warp_sum(float v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ void block_householder_qr(float* A, int m, int q, float* Rm, float* tau, float* colsc) {
-  const int p = min(m, q);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j = 0; j < p; ++j) {
-    float* x = A + (int64_t)j * m;
-    // norm of x[j+1 : m]
-    if (warp == 0) {
-      float ss = 0.f;
-      for (int i = j + 1 + lane; i < m; i += 32) ss = fmaf(x[i], x[i], ss);
-      ss = warp_sum(ss);
-      if (lane == 0) {
-        float alpha = x[j];
-        float xn = sqrtf(ss);
-        if (xn == 0.f) {
-          tau[j] = 0.f;
-          colsc[0] = 0.f;
-        } else {
-          float beta = -copysignf(hypotf(alpha, xn), alpha);
-          tau[j] = (beta - alpha) / beta;
-          colsc[0] = 1.f / (alpha - beta);
-          x[j] = beta;
-        }
-      }
-    }
-    __syncthreads();
-    const float sc = colsc[0];
-    const float tj = tau[j];
-    if (tj != 0.f)
-      for (int i = j + 1 + threadIdx.x; i < m; i += blockDim.x) x[i] *= sc;
-    __syncthreads();
-    if (tj != 0.f) {
-      // apply H_j = I - tau v v^T (v_j = 1) to columns j+1..q-1, one warp per column
-      for (int cc = j + 1 + warp; cc < q; cc += nw) {
-        float* y = A + (int64_t)cc * m;
-        float w = 0.f;
-        for (int i = j + 1 + lane; i < m; i += 32) w = fmaf(x[i], y[i], w);
-        w = warp_sum(w) + y[j];
-        w *= tj;
-        if (lane == 0) y[j] -= w;
-        for (int i = j + 1 + lane; i < m; i += 32) y[i] = fmaf(-w, x[i], y[i]);
-      }
-    }
-    __syncthreads();
-  }
-  // R (upper trapezoid) out, zero below
-  for (int idx = threadIdx.x; idx < q * q; idx += blockDim.x) {
-    int i = idx / q, jj = idx - i * q;
-    Rm[idx] = (i < p && jj >= i) ? A[(int64_t)jj * m + i] : 0.f;
-  }
-  __syncthreads();
-  // form Q in place (backward accumulation of the reflectors), columns 0..p-1
-  for (int j = p - 1; j >= 0; --j) {
-    float* x = A + (int64_t)j * m;
-    const float tj = tau[j];
-    for (int cc = j + 1 + warp; cc < p; cc += nw) {
-      float* y = A + (int64_t)cc * m;
-      float w = 0.f;
-      for (int i = j + 1 + lane; i < m; i += 32) w = fmaf(x[i], y[i], w);
-      w = (warp_sum(w) + y[j]) * tj;
-      if (lane == 0) y[j] -= w;
-      for (int i = j + 1 + lane; i < m; i += 32) y[i] = fmaf(-w, x[i], y[i]);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      if (i < j)
-        x[i] = 0.f;
-      else if (i == j)
-        x[i] = 1.f - tj;
-      else
-        x[i] = -tj * x[i];
-    }
-    __syncthreads();
-  }
-  // non-negative diagonal of R
-  for (int j = 0; j < p; ++j) {
-    if (Rm[j * q + j] < 0.f) {
-      for (int t = threadIdx.x; t < q; t += blockDim.x) Rm[j * q + t] = -Rm[j * q + t];
-      for (int i = threadIdx.x; i < m; i += blockDim.x) A[(int64_t)j * m + i] = -A[(int64_t)j * m + i];
-    }
-    __syncthreads();
-  }
-}
+// QR / LQ of cores that the kernels of tt_qr.cu do not take (ranks above 32, unfoldings beyond their
+// shared memory)
 
 // CholeskyQR2 of the m x q column-major matrix A (pitch lda) in shared memory: two passes of
 // W = A^T A (threads own (i, j, row-group) partial sums), W = R^T R (one warp, FP32 Cholesky),
@@ -904,435 +814,6 @@ __global__ void __launch_bounds__(512) k_lq_right(float* prev, float* core, int 
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// CholeskyQR2 with rows in registers, for q <= 16 columns (Q = q rounded up to 4, 8, 12 or 16),
-// 256 threads. A (m x Q, row-major, pitch QP) is in shared memory; thread t owns rows t, t + 256,
-// ... Per pass: every thread sums the outer products a a^T of its rows (Q (Q+1) / 2 packed
-// lower-triangle values in registers); each warp folds its 32 copies with a reduce-scatter of
-// shuffles (each step halves the values a lane holds), the 8 warp sums are added in a fixed
-// order; every thread then factors W = L L^T itself (FP32 Cholesky, so no further barrier) and
-// replaces each of its rows a by the solution x of x L^T = a. Padded columns (q <= j < Q) are
-// zero and get a unit pivot, so they stay zero. A pivot <= 1e-6 times the largest diagonal entry
-// of W (condition number above ~1e3, rank deficiency) returns false: the caller falls back to
-// Householder. On success Rm (q x q row-major) holds R = L_2^T L_1^T.
-
-constexpr int QR_T = 256;
-
-template <int Q>
-struct QrShape {
-  static constexpr int QP = (Q % 8 == 0) ? Q + 4 : Q;  // row pitch: conflict-free 16-byte loads
-  static constexpr int V = Q * (Q + 1) / 2;            // packed lower triangle, p = i (i+1)/2 + j
-};
-
-// Sum v[0..V) over the 32 lanes of a warp; on return lane `lane` holds the sums of the packed
-// indices base + k, k < kept (written to out[base + k] for base + k < V).
-// One step of the fold: N values per lane become H = (N + 1) / 2; a lane with the OFF bit set
-// keeps the upper half (and adds H to its base index), its partner the lower half. `cnt` counts
-// the leading slots that hold real indices; the rest are zero padding (odd N), which must not be
-// stored: their index belongs to another lane.
-template <int N, int OFF, int V>
-__device__ __forceinline__ void warp_fold_step(float (&v)[V], int lane, int& base, int& cnt) {
-  constexpr int H = (N + 1) / 2;
-  const bool up = (lane & OFF) != 0;
-#pragma unroll
-  for (int k = 0; k < H; ++k) {
-    const float lo = v[k];
-    const float hi = (H + k < N) ? v[H + k] : 0.f;
-    const float got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, OFF);
-    v[k] = (up ? hi : lo) + got;
-  }
-  if (up) {
-    base += H;
-    cnt = max(cnt - H, 0);
-  } else {
-    cnt = min(cnt, H);
-  }
-}
-
-// Sum v[0..V) over the 32 lanes of a warp (a reduce-scatter: 5 steps, each halving the values a
-// lane holds) and store the sums to out[0..V): lane `lane` ends with indices base + k.
-template <int V>
-__device__ __forceinline__ void warp_fold_store(float (&v)[V], float* out) {
-  const int lane = threadIdx.x & 31;
-  int base = 0, cnt = V;
-  constexpr int N1 = (V + 1) / 2, N2 = (N1 + 1) / 2, N3 = (N2 + 1) / 2, N4 = (N3 + 1) / 2, N5 = (N4 + 1) / 2;
-  warp_fold_step<V, 16>(v, lane, base, cnt);
-  warp_fold_step<N1, 8>(v, lane, base, cnt);
-  warp_fold_step<N2, 4>(v, lane, base, cnt);
-  warp_fold_step<N3, 2>(v, lane, base, cnt);
-  warp_fold_step<N4, 1>(v, lane, base, cnt);
-#pragma unroll
-  for (int k = 0; k < N5; ++k)
-    if (k < cnt) out[base + k] = v[k];
-}
-
-template <int Q>
-__device__ __forceinline__ void qr_load_row(const float* As, int r, float (&a)[Q]) {
-  const float4* p = reinterpret_cast<const float4*>(As + (size_t)r * QrShape<Q>::QP);
-#pragma unroll
-  for (int u = 0; u < Q / 4; ++u) {
-    const float4 x = p[u];
-    a[4 * u] = x.x;
-    a[4 * u + 1] = x.y;
-    a[4 * u + 2] = x.z;
-    a[4 * u + 3] = x.w;
-  }
-}
-
-template <int Q>
-__device__ __forceinline__ void qr_store_row(float* As, int r, const float (&a)[Q]) {
-  float4* p = reinterpret_cast<float4*>(As + (size_t)r * QrShape<Q>::QP);
-#pragma unroll
-  for (int u = 0; u < Q / 4; ++u) p[u] = make_float4(a[4 * u], a[4 * u + 1], a[4 * u + 2], a[4 * u + 3]);
-}
-
-// Shared scratch of cholqr2_rows: part (8 x V) | Wsum (V) | Ls (2 x V)
-template <int Q>
-__device__ bool cholqr2_rows(float* As, int m, int q, float* scratch, float* Rm) {
-  constexpr int V = QrShape<Q>::V;
-  float* part = scratch;
-  float* Wsum = part + 8 * V;
-  float* Ls = Wsum + V;
-  const int t = threadIdx.x, warp = t >> 5;
-  for (int pass = 0; pass < 2; ++pass) {
-    float acc[V];
-#pragma unroll
-    for (int p = 0; p < V; ++p) acc[p] = 0.f;
-    for (int r = t; r < m; r += QR_T) {
-      float a[Q];
-      qr_load_row<Q>(As, r, a);
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {  // row i of the packed triangle: pairs (j, j+1) per fma.rn.f32x2
-        const int pi = i * (i + 1) / 2;
-        const float2 ai = make_float2(a[i], a[i]);
-#pragma unroll
-        for (int j = 0; j + 1 <= i; j += 2) {
-          const float2 d = tt_ffma2(ai, make_float2(a[j], a[j + 1]), make_float2(acc[pi + j], acc[pi + j + 1]));
-          acc[pi + j] = d.x;
-          acc[pi + j + 1] = d.y;
-        }
-        if ((i & 1) == 0) acc[pi + i] = fmaf(a[i], a[i], acc[pi + i]);  // odd count: the diagonal alone
-      }
-    }
-    warp_fold_store<V>(acc, part + warp * V);
-    __syncthreads();
-    if (t < V) {
-      float sum = 0.f;
-#pragma unroll
-      for (int u = 0; u < QR_T / 32; ++u) sum += part[u * V + t];
-      Wsum[t] = sum;
-    }
-    __syncthreads();
-    float L[V], dinv[Q];
-    float dmax = 0.f;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) dmax = fmaxf(dmax, i < q ? Wsum[i * (i + 1) / 2 + i] : 0.f);
-    bool ok = dmax > 0.f && isfinite(dmax);
-#pragma unroll
-    for (int j = 0; j < Q; ++j) {
-      const int pj = j * (j + 1) / 2;
-      float d = (j < q) ? Wsum[pj + j] : 1.f;
-#pragma unroll
-      for (int l = 0; l < Q; ++l)
-        if (l < j) d = fmaf(-L[pj + l], L[pj + l], d);
-      if (j < q && (!(d > 1e-6f * dmax) || !isfinite(d))) ok = false;
-      const float ljj = sqrtf(fmaxf(d, 1e-30f));
-      L[pj + j] = ljj;
-      dinv[j] = 1.f / ljj;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        if (i <= j) continue;
-        const int pi = i * (i + 1) / 2;
-        float v = (i < q && j < q) ? Wsum[pi + j] : 0.f;
-#pragma unroll
-        for (int l = 0; l < Q; ++l)
-          if (l < j) v = fmaf(-L[pi + l], L[pj + l], v);
-        L[pi + j] = v * dinv[j];
-      }
-    }
-    if (!ok) return false;  // the same values in every thread: a uniform exit
-    for (int r = t; r < m; r += QR_T) {
-      float a[Q];
-      qr_load_row<Q>(As, r, a);
-#pragma unroll
-      for (int j = 0; j < Q; ++j) {
-        const int pj = j * (j + 1) / 2;
-        float v = a[j];
-#pragma unroll
-        for (int l = 0; l < Q; ++l)
-          if (l < j) v = fmaf(-a[l], L[pj + l], v);
-        a[j] = v * dinv[j];
-      }
-      qr_store_row<Q>(As, r, a);
-    }
-    if (t == 0) {
-#pragma unroll
-      for (int p = 0; p < V; ++p) Ls[pass * V + p] = L[p];
-    }
-  }
-  __syncthreads();
-  // R = R_2 R_1, R_p = L_p^T: R[i][j] = sum_{l = i..j} L_2[l][i] L_1[j][l]
-  for (int e = t; e < q * q; e += QR_T) {
-    const int i = e / q, j = e - i * q;
-    float acc = 0.f;
-    for (int l = i; l <= j; ++l) acc = fmaf(Ls[V + l * (l + 1) / 2 + i], Ls[j * (j + 1) / 2 + l], acc);
-    Rm[e] = acc;
-  }
-  __syncthreads();
-  return true;
-}
-
-
-// Shared-memory layout of k_qr_left_rows / k_lq_right_rows (floats): As (m x QP) | NX (the
-// neighbour core, when prefetched) | scratch (8 V + 3 V) | Rm (q x q) | tau (Q) | colsc (4)
-template <int Q>
-static size_t qr_rows_smem(int m, int64_t nx) {
-  constexpr int V = QrShape<Q>::V;
-  return sizeof(float) * ((size_t)m * QrShape<Q>::QP + (size_t)nx + 11 * V + Q * Q + Q + 4);
-}
-
-// G_k^L (m = r0 n rows, q = r1 <= Q cols) = Q R; G_k <- Q; G_{k+1} <- R G_{k+1}^R. The
-// neighbour G_{k+1} (r1 x ncols_next) is prefetched with cp.async while the QR runs when
-// `prefetch` is set (the launcher reserved room for it).
-template <int Q>
-__global__ void __launch_bounds__(QR_T, 1) k_qr_left_rows(float* core, float* next, int r0, int n, int r1,
-                                                      int ncols_next, int prefetch, const int* status) {
-  extern __shared__ __align__(16) float sm[];
-  constexpr int QP = QrShape<Q>::QP, V = QrShape<Q>::V;
-  if (*status != 0) return;
-  const int m = r0 * n, q = r1, t = threadIdx.x;
-  const int64_t nx = prefetch ? (int64_t)r1 * ncols_next : 0;
-  float* As = sm;
-  float* NX = As + (size_t)m * QP;
-  float* scratch = NX + nx;
-  float* Rm = scratch + 11 * V;
-  float* tau = Rm + Q * Q;
-  float* colsc = tau + Q;
-  bool ok = false;
-  if (m >= q) {
-    for (int j = 0; j < q; ++j)  // G_k^L column-major -> rows
-      for (int r = t; r < m; r += QR_T) cp_async4(As + (size_t)r * QP + j, core + (size_t)j * m + r);
-  }
-  cp_async_commit();  // group 0: the matrix (empty when m < q)
-  for (int64_t idx = t; idx < nx; idx += QR_T) cp_async4(NX + idx, next + idx);
-  cp_async_commit();  // group 1: the neighbour core
-  if (m >= q) {
-    for (int r = t; r < m; r += QR_T)  // zero padding columns
-#pragma unroll
-      for (int j = 0; j < QP; ++j)
-        if (j >= q) As[(size_t)r * QP + j] = 0.f;
-    cp_async_wait<1>();
-    __syncthreads();
-    ok = cholqr2_rows<Q>(As, m, q, scratch, Rm);
-    if (ok)
-      for (int j = 0; j < q; ++j)
-        for (int r = t; r < m; r += QR_T) core[(size_t)j * m + r] = As[(size_t)r * QP + j];
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  if (!ok) {  // Householder on a dense column-major copy (pitch m)
-    stage_batched(m * q, [&](int idx) { return core + idx; }, [&](int idx) { return As + idx; });
-    __syncthreads();
-    block_householder_qr(As, m, q, Rm, tau, colsc);
-    const int p = min(m, q);
-    for (int idx = t; idx < m * q; idx += QR_T) core[idx] = (idx / m < p) ? As[idx] : 0.f;
-    __syncthreads();
-  }
-  // G_{k+1}^R <- R G_{k+1}^R (r1 x ncols_next, column-major): one thread per column, the upper
-  // triangle of R in registers
-  float R[QrShape<Q>::V];
-#pragma unroll
-  for (int a2 = 0; a2 < Q; ++a2)
-#pragma unroll
-    for (int b = 0; b < Q; ++b)
-      if (b >= a2) R[b * (b + 1) / 2 + a2] = (a2 < q && b < q) ? Rm[a2 * q + b] : 0.f;
-  // with the neighbour prefetched, each thread overwrites its own columns of the shared copy and
-  // the CTA then stores the copy with coalesced writes (columns are r1 floats apart)
-  float* dstc = prefetch ? NX : next;
-  for (int cc = t; cc < ncols_next; cc += QR_T) {
-    float x[Q];
-    const float* src = prefetch ? NX + (size_t)cc * r1 : next + (size_t)cc * r1;
-#pragma unroll
-    for (int b = 0; b < Q; ++b) x[b] = b < q ? src[b] : 0.f;
-#pragma unroll
-    for (int a2 = 0; a2 < Q; ++a2) {
-      if (a2 >= q) break;
-      float acc = 0.f;
-#pragma unroll
-      for (int b = 0; b < Q; ++b)
-        if (b >= a2) acc = fmaf(R[b * (b + 1) / 2 + a2], x[b], acc);
-      dstc[(size_t)cc * r1 + a2] = acc;
-    }
-  }
-  if (prefetch) {
-    __syncthreads();
-    const int64_t nx = (int64_t)r1 * ncols_next;
-    for (int64_t idx = t; idx < nx; idx += QR_T) next[idx] = NX[idx];
-  }
-}
-
-// (G_k^R)^T (m = n r1 rows, q = r0 <= Q cols) = Q R; G_k^R <- Q^T; G_{k-1}^L <- G_{k-1}^L R^T.
-// The neighbour G_{k-1} (nrows_prev x r0) is prefetched as in k_qr_left_rows.
-template <int Q>
-__device__ void lq_right_body(float* sm, float* prev, float* core, int r0, int n, int r1, int nrows_prev,
-                              int prefetch) {
-  constexpr int QP = QrShape<Q>::QP, V = QrShape<Q>::V;
-  const int m = n * r1, q = r0, t = threadIdx.x;
-  const int64_t nx = prefetch ? (int64_t)nrows_prev * r0 : 0;
-  float* As = sm;
-  float* NX = As + (size_t)m * QP;
-  float* scratch = NX + nx;
-  float* Rm = scratch + 11 * V;
-  float* tau = Rm + Q * Q;
-  float* colsc = tau + Q;
-  bool ok = false;
-  if (m >= q) {
-    for (int i = t; i < m; i += QR_T)  // row i of (G_k^R)^T = core[q i .. q i + q)
-#pragma unroll
-      for (int a2 = 0; a2 < Q; ++a2)
-        if (a2 < q) cp_async4(As + (size_t)i * QP + a2, core + (size_t)i * q + a2);
-  }
-  cp_async_commit();  // group 0: the matrix (empty when m < q)
-  for (int64_t idx = t; idx < nx; idx += QR_T) cp_async4(NX + idx, prev + idx);
-  cp_async_commit();  // group 1: the neighbour core
-  if (m >= q) {
-    for (int r = t; r < m; r += QR_T)  // zero padding columns
-#pragma unroll
-      for (int j = 0; j < QP; ++j)
-        if (j >= q) As[(size_t)r * QP + j] = 0.f;
-    cp_async_wait<1>();
-    __syncthreads();
-    ok = cholqr2_rows<Q>(As, m, q, scratch, Rm);
-    if (ok)
-      for (int i = t; i < m; i += QR_T)
-#pragma unroll
-        for (int a2 = 0; a2 < Q; ++a2)
-          if (a2 < q) core[(size_t)i * q + a2] = As[(size_t)i * QP + a2];
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  if (!ok) {
-    stage_batched(m * q, [&](int idx) { return core + (idx / m) + (int64_t)r0 * (idx % m); },
-                  [&](int idx) { return As + idx; });  // dense, pitch m
-    __syncthreads();
-    block_householder_qr(As, m, q, Rm, tau, colsc);
-    const int p = min(m, q);
-    for (int idx = t; idx < m * q; idx += QR_T) {
-      const int i = idx % m, a2 = idx / m;
-      core[a2 + (int64_t)r0 * i] = (a2 < p) ? As[idx] : 0.f;
-    }
-    __syncthreads();
-  }
-  // G_{k-1}^L <- G_{k-1}^L R^T (nrows_prev x r0, column-major): one thread per row, the upper
-  // triangle of R in registers
-  float R[QrShape<Q>::V];
-#pragma unroll
-  for (int b = 0; b < Q; ++b)
-#pragma unroll
-    for (int a2 = 0; a2 < Q; ++a2)
-      if (a2 >= b) R[a2 * (a2 + 1) / 2 + b] = (a2 < q && b < q) ? Rm[b * q + a2] : 0.f;
-  for (int tt = t; tt < nrows_prev; tt += QR_T) {
-    float x[Q];
-    const float* src = prefetch ? NX : prev;
-#pragma unroll
-    for (int a2 = 0; a2 < Q; ++a2) x[a2] = a2 < q ? src[tt + (size_t)nrows_prev * a2] : 0.f;
-#pragma unroll
-    for (int b = 0; b < Q; ++b) {
-      if (b >= q) break;
-      float acc = 0.f;
-#pragma unroll
-      for (int a2 = 0; a2 < Q; ++a2)
-        if (a2 >= b) acc = fmaf(x[a2], R[a2 * (a2 + 1) / 2 + b], acc);
-      prev[tt + (size_t)nrows_prev * b] = acc;
-    }
-  }
-}
-
-template <int Q>
-__global__ void __launch_bounds__(QR_T, 1) k_lq_right_rows(float* prev, float* core, int r0, int n, int r1,
-                                                       int nrows_prev, int prefetch, const int* status) {
-  extern __shared__ __align__(16) float sm[];
-  if (*status != 0) return;
-  lq_right_body<Q>(sm, prev, core, r0, n, r1, nrows_prev, prefetch);
-}
-
-// The right-to-left orthogonalisation of Algorithm 1 (k = d-1 .. 1) in one CTA: each step is the
-// body of k_lq_right_rows on the cores left by the previous one (a barrier between the steps).
-struct LqSweepArgs {
-  float* core[TT_MAX_D];
-  int r[TT_MAX_D + 1];
-  int n[TT_MAX_D];
-  int d;
-  int prefetch;
-};
-
-template <int Q>
-__global__ void __launch_bounds__(QR_T, 1) k_lq_sweep_rows(LqSweepArgs a, const int* status) {
-  extern __shared__ __align__(16) float sm[];
-  if (*status != 0) return;
-  for (int k = a.d - 1; k >= 1; --k) {
-    lq_right_body<Q>(sm, a.core[k - 1], a.core[k], a.r[k], a.n[k], a.r[k + 1], a.r[k - 1] * a.n[k - 1], a.prefetch);
-    __syncthreads();
-  }
-}
-
-template <int Q>
-static bool launch_lq_sweep_q(tt_ctx* c, float* const* cores, cudaError_t* err) {
-  LqSweepArgs a;
-  a.d = c->d;
-  size_t with = 0, without = 0;
-  for (int k = 0; k < c->d; ++k) {
-    a.core[k] = cores[k];
-    a.n[k] = (int)c->n[k];
-  }
-  for (int k = 0; k <= c->d; ++k) a.r[k] = c->r[k];
-  for (int k = c->d - 1; k >= 1; --k) {
-    const int m = (int)c->n[k] * c->r[k + 1];
-    const int64_t nx = (int64_t)c->r[k - 1] * c->n[k - 1] * c->r[k];
-    with = std::max(with, qr_rows_smem<Q>(m, nx));
-    without = std::max(without, qr_rows_smem<Q>(m, 0));
-  }
-  a.prefetch = with <= 200 * 1024;
-  const size_t smem = a.prefetch ? with : without;
-  if (smem > 200 * 1024) return false;
-  *err = cudaFuncSetAttribute(k_lq_sweep_rows<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (*err != cudaSuccess) return true;
-  k_lq_sweep_rows<Q><<<1, QR_T, smem, c->stream>>>(a, c->d_status);
-  *err = cudaGetLastError();
-  return true;
-}
-
-// Launch a rows kernel for q <= 16 when its shared memory fits; false = use the generic kernels.
-template <int Q, bool LEFT>
-static bool launch_qr_rows_q(float* a0, float* a1, int r0, int n, int r1, int nbr, int m, int64_t nx,
-                             const int* status, cudaStream_t st, cudaError_t* err) {
-  size_t smem = qr_rows_smem<Q>(m, nx);
-  int prefetch = 1;
-  if (smem > 200 * 1024) {
-    prefetch = 0;
-    smem = qr_rows_smem<Q>(m, 0);
-    if (smem > 200 * 1024) return false;
-  }
-  auto kern = LEFT ? k_qr_left_rows<Q> : k_lq_right_rows<Q>;
-  *err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (*err != cudaSuccess) return true;
-  kern<<<1, QR_T, smem, st>>>(a0, a1, r0, n, r1, nbr, prefetch, status);
-  *err = cudaGetLastError();
-  return true;
-}
-
-template <bool LEFT>
-static bool launch_qr_rows(float* a0, float* a1, int r0, int n, int r1, int nbr, const int* status,
-                           cudaStream_t st, cudaError_t* err) {
-  const int q = LEFT ? r1 : r0, m = LEFT ? r0 * n : n * r1;
-  const int64_t nx = (int64_t)nbr * q;
-  if (q <= 4) return launch_qr_rows_q<4, LEFT>(a0, a1, r0, n, r1, nbr, m, nx, status, st, err);
-  if (q <= 8) return launch_qr_rows_q<8, LEFT>(a0, a1, r0, n, r1, nbr, m, nx, status, st, err);
-  if (q <= 12) return launch_qr_rows_q<12, LEFT>(a0, a1, r0, n, r1, nbr, m, nx, status, st, err);
-  if (q <= 16) return launch_qr_rows_q<16, LEFT>(a0, a1, r0, n, r1, nbr, m, nx, status, st, err);
-  return false;
-}
-
 static size_t qr_smem(int m, int q, int use_chol) {
   const size_t lda = use_chol ? (size_t)(m | 1) : (size_t)m;
   return sizeof(float) * (lda * q + (size_t)q * q + q + 4 + (size_t)std::max(q * q, 512) + (size_t)q * q);
@@ -1342,9 +823,9 @@ int tt_launch_qr_left(tt_ctx* c, float* core_k, float* core_k1, int k) {
   int r0 = c->r[k], n = (int)c->n[k], r1 = c->r[k + 1];
   int ncols = (int)(c->n[k + 1] * c->r[k + 2]);
   cudaError_t e = cudaSuccess;
-  if (launch_qr_rows<true>(core_k, core_k1, r0, n, r1, ncols, c->d_status, c->stream, &e)) {
+  if (tt_qr_left_tiles(c, core_k, core_k1, k, &e)) {
     TT_CUDA(c, e);
-    TT_LAUNCH(c, "k_qr_left_rows");
+    TT_LAUNCH(c, "k_qr_left_tiles");
     return TT_OK;
   }
   const int use_chol = (r1 <= 32) ? 1 : 0;
@@ -1355,39 +836,27 @@ int tt_launch_qr_left(tt_ctx* c, float* core_k, float* core_k1, int k) {
   return TT_OK;
 }
 
-// Right-to-left orthogonalisation of all cores: one launch when every rank r_1 .. r_{d-1} is at
-// most 16 (and shared memory allows), else one launch per step.
+// Right-to-left orthogonalisation of all cores: one launch where the kernel of tt_qr.cu takes every
+// step, else one launch per step.
 int tt_launch_lq_sweep(tt_ctx* c, float* const* cores) {
-  int q = 1;
-  for (int k = 1; k < c->d; ++k) q = std::max(q, c->r[k]);
   cudaError_t e = cudaSuccess;
-  bool done = false;
-  if (c->d >= 2 && q <= 16) {
-    if (q <= 4)
-      done = launch_lq_sweep_q<4>(c, cores, &e);
-    else if (q <= 8)
-      done = launch_lq_sweep_q<8>(c, cores, &e);
-    else if (q <= 12)
-      done = launch_lq_sweep_q<12>(c, cores, &e);
-    else
-      done = launch_lq_sweep_q<16>(c, cores, &e);
-  }
-  if (done) {
+  if (tt_lq_tiles(c, cores, c->d - 1, 1, &e)) {
     TT_CUDA(c, e);
-    TT_LAUNCH(c, "k_lq_sweep_rows");
+    TT_LAUNCH(c, "k_lq_tiles");
     return TT_OK;
   }
-  for (int kk = c->d - 1; kk >= 1; --kk) TT_TRY(tt_launch_lq_right(c, cores[kk - 1], cores[kk], kk));
+  for (int k = c->d - 1; k >= 1; --k) TT_TRY(tt_launch_lq_right(c, cores, k));
   return TT_OK;
 }
 
-int tt_launch_lq_right(tt_ctx* c, float* core_km1, float* core_k, int k) {
+int tt_launch_lq_right(tt_ctx* c, float* const* cores, int k) {
+  float *core_km1 = cores[k - 1], *core_k = cores[k];
   int r0 = c->r[k], n = (int)c->n[k], r1 = c->r[k + 1];
   int nrows = (int)(c->r[k - 1] * c->n[k - 1]);
   cudaError_t e = cudaSuccess;
-  if (launch_qr_rows<false>(core_km1, core_k, r0, n, r1, nrows, c->d_status, c->stream, &e)) {
+  if (tt_lq_tiles(c, cores, k, k, &e)) {
     TT_CUDA(c, e);
-    TT_LAUNCH(c, "k_lq_right_rows");
+    TT_LAUNCH(c, "k_lq_tiles");
     return TT_OK;
   }
   const int use_chol = (r0 <= 32) ? 1 : 0;

@@ -8,11 +8,20 @@ tolerance is the suite's for FP32 sums (1e-5 relative)."""
 import numpy as np
 import pytest
 
-torch = pytest.importorskip("torch")
-import tt_oracle as O  # noqa: E402
-from paper_2309_08093_gb300 import lib, synth  # noqa: E402
+import tt_oracle as O
+from paper_2309_08093_gb300 import synth
 
 pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2309_08093_gb300 import build as _build  # noqa: E402
+
+_build.build()
+from paper_2309_08093_gb300 import lib  # noqa: E402
+
 TOL = 1e-5
 
 SHAPES = [  # dims, J

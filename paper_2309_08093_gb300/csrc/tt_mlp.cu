@@ -9,13 +9,18 @@
 //                     "empty" mbarrier. Four stages: a stage is refilled as soon as its MMAs
 //                     released it. The
 //                     epilogue reads the accumulator with tcgen05.ld (warp w owns lanes 32w..32w+31)
-//                     and applies one of three fused epilogues:
-//                       EPI_F32   : C (+ bias) -> FP32
+//                     and applies one of four fused epilogues:
+//                       EPI_F32   : C (+ bias) -> FP32, through shared memory so that a warp stores
+//                                   128 contiguous bytes of a row (a row per lane left 4-byte pieces of
+//                                   32 rows per store: 94 us for the 256 x 23232 output layer)
+//                       EPI_LOSS  : Y = C + bias, dY = 2 (Y - T) / (B out) -> BF16 row-major and
+//                                   transposed, column sums of dY per 32 rows, the squared-error sum;
+//                                   Y and dY never reach memory in FP32
 //                       EPI_GELU  : Z = C + bias -> FP32 (kept for the backward pass),
 //                                   H = GELU(Z) -> BF16 row-major and BF16 transposed
 //                       EPI_DGELU : dZ = C * GELU'(Z) -> FP32, BF16 row-major, BF16 transposed
 //   k_input         : gather rows of X, round to BF16 (row-major and transposed), zero padding
-//   k_loss          : dY = 2 (Y - T) / (B out) and the squared-error sum (FP64)
+//   k_loss          : dY and the squared-error sum (FP64) where the output layer is split over K
 //   k_colsum        : bias gradients (column sums, fixed order)
 //   k_adam          : Adam update of FP32 masters, BF16 copies (and transposed copies)
 //
@@ -37,18 +42,24 @@
 #include "../../include/tt_warmstart.h"
 #include "tt_tc.cuh"
 
+int tt_sm_count();  // tt_context.cu
+
 namespace {
 
 typedef __nv_bfloat16 bf16;
 
 constexpr int GM = 128, GK = 64, GSTAGES = 4;  // tile N (BN) is 128 or 256, per launch
+constexpr int GT = 256;  // threads: two warps per 32 accumulator lanes share the epilogue's columns
 constexpr int A_STAGE = GM * GK * 2;  // bytes per stage of A
 template <int BN>
 constexpr int b_stage() { return BN * GK * 2; }
-template <int BN>
-constexpr int gemm_smem() { return GSTAGES * (A_STAGE + b_stage<BN>()) + 1024 + 128; }
+constexpr int WBUF = 32 * 33;  // floats of a warp's epilogue block
+template <int EPI, int BN>
+constexpr int gemm_smem() {
+  return GSTAGES * (A_STAGE + b_stage<BN>()) + 1024 + 128 + (EPI == 3 ? GT / 32 * WBUF * (int)sizeof(float) : 0);
+}
 
-enum { EPI_F32 = 0, EPI_GELU = 1, EPI_DGELU = 2 };
+enum { EPI_F32 = 0, EPI_GELU = 1, EPI_DGELU = 2, EPI_LOSS = 3 };
 
 struct GemmArgs {
   const bf16* A;
@@ -68,6 +79,14 @@ struct GemmArgs {
   int* err;           // device flag set to 1 when a bounded wait gave up
   int kchunk;         // split-K: columns of K per blockIdx.z (multiple of GK)
   int64_t slab;       // split-K: element offset between the FP32 outputs of consecutive splits
+  // EPI_LOSS: targets (row stride ldtg), row selection, valid rows and columns, 1 / (batch out), the sum;
+  // f32 receives the column sums of dY, one row (stride ldf) per 32 rows
+  const float* T;
+  int ldtg;
+  const int* rows;
+  int batch, out;
+  float inv;
+  double* loss;
 };
 
 using namespace ttc;
@@ -83,8 +102,13 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
 
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+}
+
 template <int EPI, int BN>
-__global__ void __launch_bounds__(128, 1) k_gemm_tn(const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(GT, 1) k_gemm_tn(const __grid_constant__ CUtensorMap tmA,
                                                     const __grid_constant__ CUtensorMap tmB, GemmArgs g) {
   constexpr int B_STAGE = b_stage<BN>();
   constexpr uint32_t TMEM_COLS = BN;  // the 128 x BN FP32 accumulator
@@ -122,6 +146,26 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tn(const __grid_constant__ CUte
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
   const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
+
+  const int quad = warp & 3, cbeg = (warp >> 2) * (BN / 2);  // this warp's accumulator lanes and columns
+  // EPI_LOSS: asynchronous copies of the targets of the warp's 32 x 32 block at column c0, into two
+  // buffers in turn (one past the stages, one in them); the first block's go out before the main loop.
+  // Through shared memory and rolled loops: kept in registers, the unrolled code that reads them runs
+  // from a cold instruction cache (77 and 135 us for the 256 x 23232 layer, now 55).
+  float* tbuf[2] = {reinterpret_cast<float*>(smem + GSTAGES * STAGE_BYTES + 128) + warp * WBUF,
+                    reinterpret_cast<float*>(sA) + (GT / 32 + warp) * WBUF};
+  auto targets = [&](int c0, float* dst) {
+    const int rb = m0 + 32 * quad, col = n0 + c0 + lane;
+#pragma unroll 4
+    for (int i = 0; i < 32; ++i) {
+      if (rb + i < g.batch && col < g.out) {
+        const int64_t src = g.rows ? (int64_t)__ldg(g.rows + rb + i) : (int64_t)(rb + i);
+        cp_async4(dst + i * 33 + lane, g.T + src * g.ldtg + col);
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  if constexpr (EPI == EPI_LOSS) targets(cbeg, tbuf[0]);
 
   // One thread is producer and MMA issuer: tiles go in flight up to GSTAGES ahead; after the MMAs
   // of tile kt are issued, the stage of tile kt-1 is refilled once those MMAs have released it.
@@ -162,20 +206,75 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tn(const __grid_constant__ CUte
   tc_fence_after();
 
   if (!failed) {
-    const int row = m0 + 32 * warp + lane;
+    const int row = m0 + 32 * quad + lane;
     const bool row_ok = row < g.M;
-    for (int c0 = 0; c0 < BN; c0 += 32) {
-      if (n0 + c0 >= g.N) break;  // uniform over the CTA
+    float sq = 0.0f, sqe = 0.0f;  // EPI_LOSS: this lane's squared-error sum
+    double sqd = 0.0;
+    for (int c0 = cbeg; c0 < cbeg + BN / 2; c0 += 32) {
+      if (n0 + c0 >= g.N) break;  // uniform over the warp
       uint32_t r[32];
-      tc_ld32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, r);
+      tc_ld32(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0, r);
       const int col0 = n0 + c0;
-      if (EPI == EPI_F32) {
-        if (row_ok) {
-          float* out = g.f32 + blockIdx.z * g.slab + (int64_t)row * g.ldf + col0;
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col0 + j < g.N) out[j] = __uint_as_float(r[j]) + (g.bias ? g.bias[col0 + j] : 0.0f);
+      if (EPI == EPI_F32 || EPI == EPI_LOSS) {
+        // the warp's 32 x 32 block through shared memory (the stages are free): lanes become columns
+        float* buf = reinterpret_cast<float*>(sA) + warp * WBUF;
+        const int col = col0 + lane, rb = m0 + 32 * quad, nr = min(32, g.M - rb);
+        const bool ok = col < g.N;
+        const float b = ok && g.bias ? g.bias[col] : 0.0f;
+        const int tb = ((c0 - cbeg) >> 5) & 1;
+        if constexpr (EPI == EPI_LOSS) {  // this block's targets have landed, the next block's go out
+          asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+          if (c0 + 32 < cbeg + BN / 2) targets(c0 + 32, tbuf[tb ^ 1]);
         }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) buf[lane * 33 + j] = __uint_as_float(r[j]);
+        __syncwarp();
+        if (EPI == EPI_F32) {
+          float* out = g.f32 + blockIdx.z * g.slab + (int64_t)rb * g.ldf + col;
+          if (ok)
+#pragma unroll 8
+            for (int i = 0; i < nr; ++i) out[(int64_t)i * g.ldf] = buf[i * 33 + lane] + b;
+        } else {
+          float csum = 0.0f;
+          float* tv = tbuf[tb];
+          float bq = 0.0f, bqe = 0.0f;
+          bool fine = true;  // every square lies in the pair's range
+#pragma unroll 4
+          for (int i = 0; i < nr; ++i) {
+            float d = 0.0f;
+            if (rb + i < g.batch && col < g.out) {
+              const float res = buf[i * 33 + lane] + b - tv[i * 33 + lane];
+              // squared-error sum as an unevaluated pair of floats (exact products, two-sums): this
+              // GPU's FP64 rate would bound the epilogue
+              const float ar = fabsf(res);
+              fine = fine && ((ar > 1e-15f && ar < 1e15f) || ar == 0.0f);
+              const float q = res * res, qe = fmaf(res, res, -q), t = bq + q, bb = t - bq;
+              bqe += ((bq - (t - bb)) + (q - bb)) + qe;
+              bq = t;
+              tv[i * 33 + lane] = res;
+              d = 2.0f * res * g.inv;
+            }
+            buf[i * 33 + lane] = d;
+            csum += d;
+            if (ok) g.hb[(int64_t)(rb + i) * g.ldh + col] = __float2bfloat16_rn(d);
+          }
+          if (fine) {
+            const float t = sq + bq, bb = t - sq;
+            sqe += ((sq - (t - bb)) + (bq - bb)) + bqe;
+            sq = t;
+          } else {  // the block's residuals again, in FP64
+#pragma unroll 1
+            for (int i = 0; i < nr; ++i)
+              if (rb + i < g.batch && col < g.out) sqd += (double)tv[i * 33 + lane] * (double)tv[i * 33 + lane];
+          }
+          if (ok && nr > 0) g.f32[(int64_t)(rb >> 5) * g.ldf + col] = csum;
+          __syncwarp();
+          if (row_ok)
+#pragma unroll 8
+            for (int j = 0; j < 32; ++j)  // (N is a multiple of 64: whole blocks)
+              g.ht[(int64_t)(col0 + j) * g.ldt + row] = __float2bfloat16_rn(buf[lane * 33 + j]);
+        }
+        __syncwarp();
       } else {
         // full 32-column chunks (N % 32 == 0 is checked on the host)
         float v[32];
@@ -225,9 +324,20 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tn(const __grid_constant__ CUte
         }
       }
     }
+    if (EPI == EPI_LOSS) {
+      double acc = (double)sq + (double)sqe + sqd;
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) reinterpret_cast<double*>(tbuf[0])[0] = acc;  // the warp's own block, read to the end
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (EPI == EPI_LOSS && tid == 0 && !failed) {
+    // one atomic per CTA: adds to one address run one after the other (8 per CTA: 83 us for the layer)
+    double acc = 0.0;
+    for (int w = 0; w < GT / 32; ++w) acc += reinterpret_cast<double*>(tbuf[0] + w * WBUF)[0];
+    if (acc != 0.0) atomicAdd(g.loss, acc);
+  }
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   if (failed && tid == 0 && g.err) atomicExch(g.err, 1);
@@ -243,7 +353,15 @@ __global__ void k_splitk_epi(const float* __restrict__ ws, int nsplit, int64_t s
     const int row = r0 + y, col = c0 + threadIdx.x;
     float v = 0.0f;
     if (row < g.M && col < g.N) {
-      for (int z = 0; z < nsplit; ++z) v += ws[z * slab + (int64_t)row * g.N + col];
+      const float* w = ws + (int64_t)row * g.N + col;
+      for (int z0 = 0; z0 < nsplit; z0 += 10) {  // ten loads in flight, added in order
+        float part[10];
+#pragma unroll
+        for (int u = 0; u < 10; ++u) part[u] = z0 + u < nsplit ? __ldg(w + (z0 + u) * slab) : 0.0f;
+#pragma unroll
+        for (int u = 0; u < 10; ++u)
+          if (z0 + u < nsplit) v += part[u];
+      }
       if (EPI == EPI_F32) {
         g.f32[(int64_t)row * g.ldf + col] = v + (g.bias ? g.bias[col] : 0.0f);
       } else if (EPI == EPI_GELU) {
@@ -332,13 +450,24 @@ __global__ void k_loss(const float* __restrict__ Y, int ldy, const float* __rest
   }
 }
 
-// g[j] = sum_{row < rows} D[row * ld + j] (one thread per column, fixed order).
+// g[j] = sum_{row < rows} D[row * ld + j]: 32 columns per block, 16 threads per column over contiguous
+// slices of the rows, the slices added in order.
 __global__ void k_colsum(const float* __restrict__ D, int ld, int rows, int cols, float* __restrict__ g) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= cols) return;
+  __shared__ float part[16][33];
+  const int j = blockIdx.x * 32 + threadIdx.x, y = threadIdx.y;
+  const int r0 = rows * y / 16, r1 = rows * (y + 1) / 16;
   float s = 0.0f;
-  for (int r = 0; r < rows; ++r) s += D[(int64_t)r * ld + j];
-  g[j] = s;
+  if (j < cols)
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) s += D[(int64_t)r * ld + j];
+  part[y][threadIdx.x] = s;
+  __syncthreads();
+  if (y == 0 && j < cols) {
+    s = 0.0f;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) s += part[u][threadIdx.x];
+    g[j] = s;
+  }
 }
 
 // Adam on a rows x cols FP32 matrix (row-major, leading dimension cols), then BF16 copies:
@@ -377,14 +506,19 @@ __global__ void k_adam(float* __restrict__ w, const float* __restrict__ gr, floa
   }
 }
 
-// Copy a rows x cols block between row-major matrices of different leading dimensions.
-__global__ void k_copy2d(const float* __restrict__ src, int lds, float* __restrict__ dst, int ldd, int rows,
-                         int cols) {
-  const int64_t total = (int64_t)rows * cols;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / cols, c = i % cols;
-    dst[r * ldd + c] = src[r * lds + c];
-  }
+// Copy a rows x cols block between row-major matrices of different leading dimensions: a block per four
+// rows (grid-stride), four loads in flight per thread.
+__global__ void __launch_bounds__(256) k_copy2d(const float* __restrict__ src, int lds, float* __restrict__ dst, int ldd,
+                                                int rows, int cols) {
+  for (int r0 = 4 * blockIdx.x; r0 < rows; r0 += 4 * gridDim.x)
+    for (int c = threadIdx.x; c < cols; c += blockDim.x) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = r0 + u < rows ? __ldg(src + (int64_t)(r0 + u) * lds + c) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r0 + u < rows) dst[(int64_t)(r0 + u) * ldd + c] = v[u];
+    }
 }
 
 int roundup(int x, int m) { return (x + m - 1) / m * m; }
@@ -470,7 +604,7 @@ template <int EPI, int BN>
 int launch_tiles_bn(tt_mlp* m, const GemmArgs& g, int nsplit, cudaStream_t s) {
   static bool attr_done = false;  // per template instance; the attribute is per function
   if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem<BN>());
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem<EPI, BN>());
     if (e != cudaSuccess) return mfail(m, TT_ECUDA, "gemm smem attribute: %s", cudaGetErrorString(e));
     attr_done = true;
   }
@@ -478,17 +612,21 @@ int launch_tiles_bn(tt_mlp* m, const GemmArgs& g, int nsplit, cudaStream_t s) {
   MLP_TRY(make_tmap(m, &tmA, g.A, g.M, g.K, g.lda, GM));
   MLP_TRY(make_tmap(m, &tmB, g.B, g.N, g.K, g.ldb, BN));
   dim3 grid((g.N + BN - 1) / BN, (g.M + GM - 1) / GM, nsplit);
-  k_gemm_tn<EPI, BN><<<grid, 128, gemm_smem<BN>(), s>>>(tmA, tmB, g);
+  k_gemm_tn<EPI, BN><<<grid, GT, gemm_smem<EPI, BN>(), s>>>(tmA, tmB, g);
   MLP_LAUNCH(m, "k_gemm_tn");
   return TT_OK;
 }
 
-// 128 x 256 tiles when that still gives every SM a CTA (fewer operand re-reads per FLOP),
-// 128 x 128 otherwise
+// 128 x 256 tiles when that still gives every SM a CTA (fewer operand re-reads per FLOP), 128 x 128
+// otherwise. The loss epilogue, longer than the products before it, also takes the narrow tiles where
+// they end in fewer half waves (256 x 23232 x 512: 182 wide tiles are two waves of 152 SMs, 67 us; 364
+// narrow ones three half ones, 55 us; plain FP32 outputs are faster wide: 24 against 30 us for dW3).
 template <int EPI>
 int launch_tiles(tt_mlp* m, const GemmArgs& g, int nsplit, cudaStream_t s) {
-  const int64_t wide = (int64_t)((g.N + 255) / 256) * ((g.M + GM - 1) / GM) * nsplit;
-  if (wide >= 148) return launch_tiles_bn<EPI, 256>(m, g, nsplit, s);
+  const int64_t rows = (int64_t)((g.M + GM - 1) / GM) * nsplit, sms = tt_sm_count();
+  const int64_t wide = (g.N + 255) / 256 * rows, narrow = (g.N + 127) / 128 * rows;
+  const bool few = EPI == EPI_LOSS && (narrow + sms - 1) / sms < 2 * ((wide + sms - 1) / sms);
+  if (wide >= 148 && !few) return launch_tiles_bn<EPI, 256>(m, g, nsplit, s);
   return launch_tiles_bn<EPI, 128>(m, g, nsplit, s);
 }
 
@@ -553,7 +691,7 @@ int pack_weights(tt_mlp* m) {
   return TT_OK;
 }
 
-// forward pass for `batch` rows; leaves Z1, Z2, H*, Y in the network's buffers
+// the hidden layers for `batch` rows; leaves Z1, Z2 and H* in the network's buffers
 int forward(tt_mlp* m, const float* X, int ldx, const int* rows, int batch) {
   const int Bp = roundup(batch, 64);
   {
@@ -567,50 +705,70 @@ int forward(tt_mlp* m, const float* X, int ldx, const int* rows, int batch) {
   g = gemm_args(m->H1b, m->hid, m->W2b, m->hid, Bp, m->hid, m->hid, m->d_err);
   g.bias = m->P[3]; g.f32 = m->Z2; g.ldf = m->hid; g.hb = m->H2b; g.ldh = m->hid; g.ht = m->H2t; g.ldt = m->bmax_p;
   MLP_TRY(launch_gemm<EPI_GELU>(m, g, m->stream));
-  g = gemm_args(m->H2b, m->hid, m->W3b, m->hid, Bp, m->out_p, m->hid, m->d_err);
-  g.bias = m->P[5]; g.f32 = m->Y; g.ldf = m->out_p;
-  MLP_TRY(launch_gemm<EPI_F32>(m, g, m->stream));
   return TT_OK;
 }
 
-// loss gradient and backward pass into m->G[*]
-int backward(tt_mlp* m, const float* T, int ldt, const int* rows, int batch) {
+// column sums of a rows x cols matrix (bias gradients)
+int colsum(tt_mlp* m, const float* D, int ld, int rows, int cols, float* g) {
+  k_colsum<<<(cols + 31) / 32, dim3(32, 16), 0, m->stream>>>(D, ld, rows, cols, g);
+  MLP_LAUNCH(m, "k_colsum");
+  return TT_OK;
+}
+
+// output layer, loss and its gradient dY (dYb, dYt, the bias gradient into gb): one GEMM with the loss in
+// its epilogue; where the output layer is split over K, the layer and then k_loss
+int loss_layer(tt_mlp* m, const float* T, int ldt, const int* rows, int batch, float* gb, int gb_cols) {
   const int Bp = roundup(batch, 64);
+  const float inv = (float)(1.0 / ((double)batch * (double)m->out));
   MLP_CUDA(m, cudaMemsetAsync(m->d_loss, 0, sizeof(double), m->stream));
+  GemmArgs g = gemm_args(m->H2b, m->hid, m->W3b, m->hid, Bp, m->out_p, m->hid, m->d_err);
+  g.bias = m->P[5];
+  g.ldf = m->out_p;
+  if (choose_split(g.M, g.N, g.K, m->ws_cap) <= 1) {
+    g.f32 = m->dY; g.hb = m->dYb; g.ldh = m->out_p; g.ht = m->dYt; g.ldt = m->bmax_p;
+    g.T = T; g.ldtg = ldt; g.rows = rows; g.batch = batch; g.out = m->out; g.inv = inv; g.loss = m->d_loss;
+    MLP_TRY(launch_tiles<EPI_LOSS>(m, g, 1, m->stream));
+    return colsum(m, m->dY, m->out_p, Bp / 32, gb_cols, gb);
+  }
+  g.f32 = m->Y;
+  MLP_TRY(launch_gemm<EPI_F32>(m, g, m->stream));
   {
     dim3 grid((m->out_p + 31) / 32, (Bp + 31) / 32), blk(32, 8);
-    const float inv = (float)(1.0 / ((double)batch * (double)m->out));
     k_loss<<<grid, blk, 0, m->stream>>>(m->Y, m->out_p, T, ldt, rows, batch, m->out, m->out_p, Bp, inv, m->dY,
                                         m->dYb, m->dYt, m->bmax_p, m->d_loss);
     MLP_LAUNCH(m, "k_loss");
   }
-  // dW3 = dY^T H2, db3 = colsum(dY)
-  GemmArgs g = gemm_args(m->dYt, m->bmax_p, m->H2t, m->bmax_p, m->out_p, m->hid, Bp, m->d_err);
-  g.f32 = m->G[4]; g.ldf = m->hid;
+  return colsum(m, m->dY, m->out_p, Bp, gb_cols, gb);
+}
+
+// loss gradient and backward pass. Gradients go to gout[i] (caller's arrays, unpadded) where given, else
+// to m->G[i] (padded).
+int backward(tt_mlp* m, const float* T, int ldt, const int* rows, int batch, float* const* gout) {
+  const int Bp = roundup(batch, 64);
+  const bool own4 = !gout[4], own0 = !gout[0];
+  MLP_TRY(loss_layer(m, T, ldt, rows, batch, gout[5] ? gout[5] : m->G[5], gout[5] ? m->out : m->out_p));
+  // dW3 = dY^T H2
+  GemmArgs g = gemm_args(m->dYt, m->bmax_p, m->H2t, m->bmax_p, own4 ? m->out_p : m->out, m->hid, Bp, m->d_err);
+  g.f32 = own4 ? m->G[4] : gout[4]; g.ldf = m->hid;
   MLP_TRY(launch_gemm<EPI_F32>(m, g, m->stream));
-  k_colsum<<<(m->out_p + 255) / 256, 256, 0, m->stream>>>(m->dY, m->out_p, Bp, m->out_p, m->G[5]);
-  MLP_LAUNCH(m, "k_colsum");
   // dZ2 = (dY W3) * GELU'(Z2)
   g = gemm_args(m->dYb, m->out_p, m->W3t, m->out_p, Bp, m->hid, m->out_p, m->d_err);
   g.f32 = m->dZ2; g.ldf = m->hid; g.zin = m->Z2; g.hb = m->dZ2b; g.ldh = m->hid; g.ht = m->dZ2t; g.ldt = m->bmax_p;
   MLP_TRY(launch_gemm<EPI_DGELU>(m, g, m->stream));
   // dW2 = dZ2^T H1, db2
   g = gemm_args(m->dZ2t, m->bmax_p, m->H1t, m->bmax_p, m->hid, m->hid, Bp, m->d_err);
-  g.f32 = m->G[2]; g.ldf = m->hid;
+  g.f32 = gout[2] ? gout[2] : m->G[2]; g.ldf = m->hid;
   MLP_TRY(launch_gemm<EPI_F32>(m, g, m->stream));
-  k_colsum<<<(m->hid + 255) / 256, 256, 0, m->stream>>>(m->dZ2, m->hid, Bp, m->hid, m->G[3]);
-  MLP_LAUNCH(m, "k_colsum");
+  MLP_TRY(colsum(m, m->dZ2, m->hid, Bp, m->hid, gout[3] ? gout[3] : m->G[3]));
   // dZ1 = (dZ2 W2) * GELU'(Z1)
   g = gemm_args(m->dZ2b, m->hid, m->W2t, m->hid, Bp, m->hid, m->hid, m->d_err);
   g.f32 = m->dZ1; g.ldf = m->hid; g.zin = m->Z1; g.hb = m->dZ1b; g.ldh = m->hid; g.ht = m->dZ1t; g.ldt = m->bmax_p;
   MLP_TRY(launch_gemm<EPI_DGELU>(m, g, m->stream));
   // dW1 = dZ1^T X, db1
-  g = gemm_args(m->dZ1t, m->bmax_p, m->XbT, m->bmax_p, m->hid, m->in_p, Bp, m->d_err);
-  g.f32 = m->G[0]; g.ldf = m->in_p;
+  g = gemm_args(m->dZ1t, m->bmax_p, m->XbT, m->bmax_p, m->hid, own0 ? m->in_p : m->in, Bp, m->d_err);
+  g.f32 = own0 ? m->G[0] : gout[0]; g.ldf = own0 ? m->in_p : m->in;
   MLP_TRY(launch_gemm<EPI_F32>(m, g, m->stream));
-  k_colsum<<<(m->hid + 255) / 256, 256, 0, m->stream>>>(m->dZ1, m->hid, Bp, m->hid, m->G[1]);
-  MLP_LAUNCH(m, "k_colsum");
-  return TT_OK;
+  return colsum(m, m->dZ1, m->hid, Bp, m->hid, gout[1] ? gout[1] : m->G[1]);
 }
 
 int check_batch(tt_mlp* m, const float* X, int ldx, int batch) {
@@ -709,7 +867,7 @@ extern "C" int tt_mlp_set_weights(tt_mlp* m, const float* W1, const float* b1, c
     MLP_CUDA(m, cudaMemsetAsync(m->P[i], 0, bytes, m->stream));
     MLP_CUDA(m, cudaMemsetAsync(m->Mo[i], 0, bytes, m->stream));
     MLP_CUDA(m, cudaMemsetAsync(m->Vo[i], 0, bytes, m->stream));
-    k_copy2d<<<256, 256, 0, m->stream>>>(src[i], cols[i], m->P[i], m->pcol[i], rows[i], cols[i]);
+    k_copy2d<<<1216, 256, 0, m->stream>>>(src[i], cols[i], m->P[i], m->pcol[i], rows[i], cols[i]);
     MLP_LAUNCH(m, "k_copy2d");
   }
   m->t = 0;
@@ -723,7 +881,7 @@ extern "C" int tt_mlp_get_weights(tt_mlp* m, float* W1, float* b1, float* W2, fl
   const int rows[6] = {m->hid, 1, m->hid, 1, m->out, 1};
   const int cols[6] = {m->in, m->hid, m->hid, m->hid, m->hid, m->out};
   for (int i = 0; i < 6; ++i) {
-    k_copy2d<<<256, 256, 0, m->stream>>>(m->P[i], m->pcol[i], dst[i], cols[i], rows[i], cols[i]);
+    k_copy2d<<<1216, 256, 0, m->stream>>>(m->P[i], m->pcol[i], dst[i], cols[i], rows[i], cols[i]);
     MLP_LAUNCH(m, "k_copy2d");
   }
   return TT_OK;
@@ -735,9 +893,9 @@ extern "C" int tt_mlp_forward(tt_mlp* m, const float* X, int ldx, const int* row
   if (!Y || ldy < m->out) return mfail(m, TT_EINVAL, "bad output (ldy %d < out_dim %d or null)", ldy, m->out);
   MLP_CUDA(m, cudaMemsetAsync(m->d_err, 0, sizeof(int), m->stream));
   MLP_TRY(forward(m, X, ldx, rows, batch));
-  k_copy2d<<<256, 256, 0, m->stream>>>(m->Y, m->out_p, Y, ldy, batch, m->out);
-  MLP_LAUNCH(m, "k_copy2d");
-  return TT_OK;
+  GemmArgs g = gemm_args(m->H2b, m->hid, m->W3b, m->hid, batch, m->out, m->hid, m->d_err);
+  g.bias = m->P[5]; g.f32 = Y; g.ldf = ldy;
+  return launch_gemm<EPI_F32>(m, g, m->stream);
 }
 
 extern "C" int tt_mlp_loss_grads(tt_mlp* m, const float* X, int ldx, const float* T, int ldt, const int* rows,
@@ -748,15 +906,8 @@ extern "C" int tt_mlp_loss_grads(tt_mlp* m, const float* X, int ldx, const float
   if (!T || ldt < m->out) return mfail(m, TT_EINVAL, "bad targets (ldt %d < out_dim %d or null)", ldt, m->out);
   MLP_CUDA(m, cudaMemsetAsync(m->d_err, 0, sizeof(int), m->stream));
   MLP_TRY(forward(m, X, ldx, rows, batch));
-  MLP_TRY(backward(m, T, ldt, rows, batch));
-  float* dst[6] = {gW1, gb1, gW2, gb2, gW3, gb3};
-  const int r[6] = {m->hid, 1, m->hid, 1, m->out, 1};
-  const int c[6] = {m->in, m->hid, m->hid, m->hid, m->hid, m->out};
-  for (int i = 0; i < 6; ++i) {
-    if (!dst[i]) continue;
-    k_copy2d<<<256, 256, 0, m->stream>>>(m->G[i], m->pcol[i], dst[i], c[i], r[i], c[i]);
-    MLP_LAUNCH(m, "k_copy2d");
-  }
+  float* const dst[6] = {gW1, gb1, gW2, gb2, gW3, gb3};
+  MLP_TRY(backward(m, T, ldt, rows, batch, dst));
   MLP_TRY(check_err_flag(m));
   if (loss_out) {
     double s = 0.0;
@@ -774,7 +925,8 @@ extern "C" int tt_mlp_train_step(tt_mlp* m, const float* X, int ldx, const float
   if (!T || ldt < m->out) return mfail(m, TT_EINVAL, "bad targets (ldt %d < out_dim %d or null)", ldt, m->out);
   MLP_CUDA(m, cudaMemsetAsync(m->d_err, 0, sizeof(int), m->stream));
   MLP_TRY(forward(m, X, ldx, rows, batch));
-  MLP_TRY(backward(m, T, ldt, rows, batch));
+  float* const own[6] = {nullptr};
+  MLP_TRY(backward(m, T, ldt, rows, batch, own));
   m->t += 1;
   const double c1 = 1.0 - std::pow((double)m->b1, (double)m->t);
   const double c2 = 1.0 - std::pow((double)m->b2, (double)m->t);

@@ -12,6 +12,8 @@
 //   k_prefix_step  : L_{<j+1}(w) = L_{<j}(w) Ghat_j(w)                      (one thread per w, b)
 //   k_face_ifft2   : two columns c = a + r_k b of S H_k: inverse FFT of L_{<k}(w)[a] R_{>k}(w)[b]
 //                    (k_face_ifft, one column with radix-2, for J = 16384)
+#include <algorithm>
+
 #include "tt_internal.cuh"
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
@@ -169,7 +171,7 @@ __global__ void k_core_fft(CoreFftArgs a) {  // one fibre per CTA (pair0 counts 
 
 // Two CountSketched fibres per CTA, packed as z = x0 + i x1: one complex FFT, then
 // X0[w] = (Z[w] + conj Z[J-w]) / 2 and X1[w] = (Z[w] - conj Z[J-w]) / 2i for w <= J/2.
-__global__ void __launch_bounds__(512) k_core_fft2(CoreFftArgs a) {
+__global__ void __launch_bounds__(1024) k_core_fft2(CoreFftArgs a) {
   extern __shared__ float2 fbuf[];
   float2* x = fbuf;
   float2* y = fbuf + a.J;
@@ -213,6 +215,9 @@ __global__ void __launch_bounds__(512) k_core_fft2(CoreFftArgs a) {
   }
 }
 
+// threads of a two-transform FFT CTA: one radix-4 butterfly each per stage, up to 1024
+static int fft_threads(const tt_ctx* c) { return std::min(1024, std::max(128, (c->J / 4 + 31) & ~31)); }
+
 // FFT sketches of cores j0 .. j1-1 in one launch
 static int launch_core_ffts(tt_ctx* c, float* const* cores, int j0, int j1) {
   CoreFftArgs a;
@@ -243,7 +248,7 @@ static int launch_core_ffts(tt_ctx* c, float* const* cores, int j0, int j1) {
       TT_CUDA(c, cudaFuncSetAttribute(k_core_fft2, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (int)sizeof(float2) * 8192));
       attr = true;
     }
-    k_core_fft2<<<a.pair0[a.ncores], 512, smem, c->stream>>>(a);
+    k_core_fft2<<<a.pair0[a.ncores], fft_threads(c), smem, c->stream>>>(a);
     TT_LAUNCH(c, "k_core_fft2");
     return TT_OK;
   }
@@ -384,7 +389,7 @@ __device__ __forceinline__ void face_zero(const FaceArgs& a) {
     a.zero[i] = 0.f;
 }
 
-__global__ void __launch_bounds__(256) k_face_ifft2(FaceArgs a) {
+__global__ void __launch_bounds__(1024) k_face_ifft2(FaceArgs a) {
   extern __shared__ float2 fbuf[];
   face_zero(a);
   float2* x = fbuf;
@@ -470,7 +475,7 @@ int tt_launch_interface_from_chain(tt_ctx* c, int k, float* SH, float* zero, int
       TT_CUDA(c, cudaFuncSetAttribute(k_face_ifft2, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (int)sizeof(float2) * 8192));
       attr = true;
     }
-    k_face_ifft2<<<(a.ra * a.rb + 1) / 2, 256, smem, c->stream>>>(a);
+    k_face_ifft2<<<(a.ra * a.rb + 1) / 2, fft_threads(c), smem, c->stream>>>(a);
     TT_LAUNCH(c, "k_face_ifft2");
     return TT_OK;
   }

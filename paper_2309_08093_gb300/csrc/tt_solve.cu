@@ -978,12 +978,13 @@ __global__ void __launch_bounds__(256) k_rel_error(ErrArgs a) {
       W[(size_t)al * WP + c] = acc;
     }
     __syncthreads();
-    // tiles of 4 consecutive i0 for one i1 (when n0 % 4 == 0): one vector load of A (issued before
+    // tiles of 4 consecutive i0 for one i1 (when n0 % 4 == 0 and A lies on a 16-byte boundary, as those
+    // loads need): one vector load of A (issued before
     // the reconstruction so its latency overlaps the FMAs), one 16-byte G_0 load and one broadcast
     // W load per rank index feed 4 FMAs. Otherwise tiles of 4 consecutive i1 for one i0.
     const int64_t base = t * (int64_t)n0 * n1 + (int64_t)j0 * n0;
     float fe = 0.f, fa = 0.f;
-    if ((n0 & 3) == 0) {
+    if ((n0 & 3) == 0 && (reinterpret_cast<uintptr_t>(a.A) & 15) == 0) {
       const int q4 = n0 >> 2;
       const int tiles = q4 * (j1 - j0);
       constexpr int UT = 4;  // tiles per thread in flight
@@ -1479,7 +1480,8 @@ int tt_launch_rel_error(tt_ctx* c, const void* A, const float* scales, float* co
   const size_t smem = sizeof(float) * ((size_t)c->r[1] * a.i1chunk + (size_t)g0sz);
   TT_CUDA(c, cudaMemsetAsync(acc, 0, sizeof(double) * 2, c->stream));
   const int es = c->dtype == TT_F64 ? 8 : c->dtype == TT_F32 ? 4 : c->dtype == TT_BF16 ? 2 : 1;
-  const size_t ssm = c->d_rint ? rel_stream_smem(c, es) : 0;
+  // (the streaming form's bulk copies start on 16-byte boundaries)
+  const size_t ssm = c->d_rint && (reinterpret_cast<uintptr_t>(A) & 15) == 0 ? rel_stream_smem(c, es) : 0;
   if (ssm) {  // streaming form: right interfaces first, then one pass over A in memory order
     const int per = (int)c->n[1] * c->rint_r1p;
     const int r2 = c->r[2];

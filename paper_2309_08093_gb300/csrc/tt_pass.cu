@@ -656,6 +656,11 @@ int64_t pass_ctas(const tt_ctx* c, int per_sm) {
   return std::max<int64_t>(1, ctas);
 }
 
+// shared memory of k_tail_pass: chunk + 1 staged entries, lists, buckets, row scales
+size_t tail_smem(int64_t chunk, int64_t blocks, int64_t J, int64_t entry_bytes, int64_t nscales) {
+  return ((size_t)((chunk + 1) * entry_bytes + 15) & ~(size_t)15) + (size_t)(8 * blocks + 4 * J + 4 * nscales);
+}
+
 template <int DT, int V, int EPW>
 int launch_tail_v(tt_ctx* c, TailArgs a) {
   using Sh = TailShape<DT, V, EPW>;
@@ -663,8 +668,7 @@ int launch_tail_v(tt_ctx* c, TailArgs a) {
   a.units = (int64_t)a.nchunk * a.ngl * a.ns;
   a.parts = 1;
   while (a.parts < 8 && 2 * a.parts * a.J <= TAIL_T) a.parts *= 2;
-  const size_t smem = (((size_t)(a.chunk + 1) * Sh::ENT + 15) & ~(size_t)15) + 8 * (size_t)a.blocks + 4 * (size_t)a.J +
-                      (DT == TT_FP8E4M3 ? 4 * (size_t)a.n0 : 0);
+  const size_t smem = tail_smem(a.chunk, a.blocks, a.J, Sh::ENT, DT == TT_FP8E4M3 ? a.n0 : 0);
   void (*kern)(TailArgs) = a.J <= 1024   ? k_tail_pass<DT, V, EPW, 1>
                            : a.J <= 2048 ? k_tail_pass<DT, V, EPW, 2>
                            : a.J <= 4096 ? k_tail_pass<DT, V, EPW, 4>
@@ -748,12 +752,17 @@ void tt_pass_plan(tt_ctx* c) {
   const int nt = c->d >= 4 ? 2 : c->d == 3 ? 1 : 0;
   if (nt) {
     const int64_t E = c->stride[c->d - nt];
-    const int64_t cm = tail_chunk_max(c);
-    c->tail_nchunk = (int)((E + cm - 1) / cm);
-    c->tail_chunk = (int)(((E + c->tail_nchunk - 1) / c->tail_nchunk + 3) & ~3);
-    // a bucket's blocks: all full but its last one
-    c->tail_blocks = c->tail_chunk / 4 + std::min(c->J, c->tail_chunk);
-    c->pass_tail = E >= 512 && E * 8 >= c->J && c->tail_nchunk <= 64;
+    const bool fp8 = c->dtype == TT_FP8E4M3;
+    // the longest chunk, halved until an SM's shared memory holds it (long FP8 rows bring a scale each)
+    bool fits = false;
+    for (int64_t cm = tail_chunk_max(c); !fits && cm >= 2048; cm /= 2) {
+      c->tail_nchunk = (int)std::min<int64_t>((E + cm - 1) / cm, 65);
+      c->tail_chunk = (int)((std::min(cm, (E + c->tail_nchunk - 1) / c->tail_nchunk) + 3) & ~3);
+      // a bucket's blocks: all full but its last one
+      c->tail_blocks = c->tail_chunk / 4 + std::min(c->J, c->tail_chunk);
+      fits = tail_smem(c->tail_chunk, c->tail_blocks, c->J, fp8 ? 4 : 8, fp8 ? c->n[0] : 0) <= 227 * 1024;
+    }
+    c->pass_tail = fits && E >= 512 && E * 8 >= c->J && c->tail_nchunk <= 64;
     if (c->pass_tail) c->tail_modes = nt;
   }
   c->head_sorted = c->pass_head && c->N / e2 <= HEAD_PLAN_MAX;

@@ -39,13 +39,13 @@ SHAPES = [  # dims, J
 ]
 
 
-def _check(dims, J, dtype, offset=0, columns=None):
+def _check(dims, J, dtype, offset=0, columns=None, rank=2):
     seed = 977
     a = synth.random_tensor(dims, 31)
     flat, scales, exact = synth.quantize(a, dtype)
     A = lib.device_tensor(np.concatenate([np.zeros(offset, flat.dtype), flat]), dtype)[offset:]
     sc = torch.from_numpy(scales).cuda() if scales is not None else None
-    ctx = lib.Context(dims, [1] + [2] * (len(dims) - 1) + [1], J, 1e-3, seed, dtype)
+    ctx = lib.Context(dims, [1] + [rank] * (len(dims) - 1) + [1], J, 1e-3, seed, dtype)
     Y = [torch.full((n, J), 3.0, device="cuda") for n in dims]
     for sweep in (4, 5):  # a second draw: accumulators and plans of the first are gone
         ctx.tt_sketch_unfold(A, -1, sweep, Y, sc)
@@ -73,6 +73,12 @@ def test_all_modes_against_the_oracle(dims, J, dtype):
                                           ("fp8", 1), ("fp8", 2), ("fp8", 4), ("fp8", 8)])
 def test_tensor_off_the_16_byte_grid(dtype, offset):
     _check((32, 24, 7, 5), 256, dtype, offset)
+
+
+@pytest.mark.parametrize("n0", [6000, 24000, 40000])
+def test_fp8_row_scales_beside_the_tail_chunk(n0):
+    """A scale per row of A in shared memory: whole chunks, shorter ones, and no tail pass."""
+    _check((n0, 3, 4), 8192, "fp8", columns=3, rank=1)
 
 
 def test_more_slabs_than_one_cta_sorts():

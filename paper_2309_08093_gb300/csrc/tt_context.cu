@@ -603,11 +603,11 @@ int tt_ensure_rplan(tt_ctx* c, int k) {
 
 int tt_ensure_plan0(tt_ctx* c) { return tt_ensure_rplan(c, 0); }
 
-int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep) {
+int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep, const void* A) {
   // (the deterministic mode's plans too: tt_ensure_rplan builds them in index order)
   if (c->capture_mode || c->user_tables || (c->flags & TT_FLAG_FIXED_SKETCH)) return TT_OK;
   bool ready = c->spare.tables_valid && c->spare.tables_sweep == sweep;
-  const unsigned plans = tt_pass_plans(c);
+  const unsigned plans = tt_pass_plans(c, A);
   for (int k = 0; k < c->d; ++k) ready = ready && (c->spare.rplan_valid[k] || !(plans & (1u << k)));
   ready = ready && (c->spare.pass_valid || c->det);
   if (ready) return TT_OK;

@@ -300,7 +300,7 @@ int tt_cuda_check(tt_ctx* c, cudaError_t e, const char* what);
 int tt_ensure_tables(tt_ctx* c, uint64_t sweep);
 // Build the tables and plans of draw `sweep` into the spare on the side stream (no-op in graph
 // capture, with user tables or a fixed sketch, or when the spare already holds that draw).
-int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep);
+int tt_prepare_next_draw(tt_ctx* c, uint64_t sweep, const void* A);
 void tt_swap_draw(tt_ctx* c);
 int tt_ensure_plan0(tt_ctx* c);
 int tt_ensure_rplan(tt_ctx* c, int k);
@@ -314,8 +314,8 @@ int tt_launch_unfold_planned(tt_ctx* c, const void* A, const float* scales, int 
 // allows, tt_launch_unfold for the other modes; ev[k] (optional) is recorded after Y[k]
 int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev = nullptr);
 void tt_pass_plan(tt_ctx* c);                 // which modes the passes cover, from the shape
-unsigned tt_pass_mask(const tt_ctx* c);       // modes covered by the passes
-unsigned tt_pass_plans(const tt_ctx* c);      // modes whose fibre plan tt_launch_unfold_all reads
+unsigned tt_pass_mask(const tt_ctx* c, const void* A);   // modes of A covered by the passes
+unsigned tt_pass_plans(const tt_ctx* c, const void* A);  // modes whose fibre plan tt_launch_unfold_all reads
 int tt_launch_pass_plans(tt_ctx* c);          // d_hplan, d_rkey, d_tlist, d_tbucket of the current draw
 int tt_launch_unfold_coo(tt_ctx* c, const int32_t* idx, const float* val, int64_t nnz, int k, float* const* Y);
 // d_err_acc[0..2] = sum val^2, sum val X(i), ||X||^2 of a sparse tensor in coordinate form

@@ -418,14 +418,10 @@ struct TailShape {
   static constexpr int ENT = V * SB;  // bytes of a staged entry
 };
 
-// x + y in one instruction
-__device__ __forceinline__ float2 add2(float2 x, float2 y) {
-  float2 d;
-  asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y));
-  return d;
+// q += x for the two FP32 values of 64-bit words (add.rn.f32x2): kept in 64-bit registers, so that the
+// shared-memory load feeds the add without moves
+__device__ __forceinline__ void add2(unsigned long long& q, unsigned long long x) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(q) : "l"(x));
 }
 
 // One CTA of 1024 threads per SM; unit = (chunk, group of V indices i_l, i_s), consecutive units in one
@@ -518,10 +514,7 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
   // q += the V values of the chunk's entry number x
   auto gather = [&](uint32_t x, float (&q)[V]) {
     const unsigned char* src = buf + x * ENT;
-    if constexpr (EB >= 4) {
-      const float2 r = add2(make_float2(q[0], q[1]), *reinterpret_cast<const float2*>(src));
-      q[0] = r.x, q[1] = r.y;
-    } else if constexpr (EB == 2) {
+    if constexpr (EB == 2) {
       tt_fma_bf16x2(*reinterpret_cast<const uint32_t*>(src), 0x3F80, q[0], q[1]);
       if constexpr (V == 4) tt_fma_bf16x2(*reinterpret_cast<const uint32_t*>(src + 4), 0x3F80, q[2], q[3]);
     } else {
@@ -616,12 +609,25 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
       float q[V];
 #pragma unroll
       for (int v = 0; v < V; ++v) q[v] = 0.f;
-      for (int p = p0 + part; p < pe; p += parts) {
-        const uint2 x = sl[p];
-        gather(x.x & 0xFFFFu, q);
-        gather(x.x >> 16, q);
-        gather(x.y & 0xFFFFu, q);
-        gather(x.y >> 16, q);
+      if constexpr (EB >= 4) {
+        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(buf);
+        unsigned long long qq = 0;
+        for (int p = p0 + part; p < pe; p += parts) {
+          const uint2 x = sl[p];
+          add2(qq, src[x.x & 0xFFFFu]);
+          add2(qq, src[x.x >> 16]);
+          add2(qq, src[x.y & 0xFFFFu]);
+          add2(qq, src[x.y >> 16]);
+        }
+        q[0] = __uint_as_float((uint32_t)qq), q[1] = __uint_as_float((uint32_t)(qq >> 32));
+      } else {
+        for (int p = p0 + part; p < pe; p += parts) {
+          const uint2 x = sl[p];
+          gather(x.x & 0xFFFFu, q);
+          gather(x.x >> 16, q);
+          gather(x.y & 0xFFFFu, q);
+          gather(x.y >> 16, q);
+        }
       }
       if (parts > 1)
 #pragma unroll
@@ -730,8 +736,18 @@ int head_cols(const tt_ctx* c) {  // columns i_1 per chunk
   return (int)(((c->n[1] + nch - 1) / nch + 3) & ~3);
 }
 
-// entries per chunk: what a CTA's threads can fetch at once (JJ loads each; the narrow loads' reach)
-int64_t tail_chunk_max(const tt_ctx* c) { return c->dtype == TT_F64 ? TAIL_T * 5 : TAIL_T * 10; }
+// entries per chunk: what a CTA's threads can fetch at once (JJ loads each). FP8 slabs on 4-byte
+// boundaries come four entries to a load; the other narrow types keep to what entry loads reach too.
+int64_t tail_chunk_max(const tt_ctx* c, int64_t E) {
+  if (c->dtype == TT_F64) return TAIL_T * 5;
+  return c->dtype == TT_FP8E4M3 && E % 4 == 0 ? TAIL_T * 20 : TAIL_T * 10;
+}
+
+// whether the tail pass can take this A: chunks sized for four entries to a load need its base on a
+// 4-byte boundary
+bool tail_takes(const tt_ctx* c, const void* A) {
+  return c->pass_tail && (c->tail_chunk <= TAIL_T * 10 || reinterpret_cast<uintptr_t>(A) % 4 == 0);
+}
 
 }  // namespace
 
@@ -755,7 +771,7 @@ void tt_pass_plan(tt_ctx* c) {
     const bool fp8 = c->dtype == TT_FP8E4M3;
     // the longest chunk, halved until an SM's shared memory holds it (long FP8 rows bring a scale each)
     bool fits = false;
-    for (int64_t cm = tail_chunk_max(c); !fits && cm >= 2048; cm /= 2) {
+    for (int64_t cm = tail_chunk_max(c, E); !fits && cm >= 2048; cm /= 2) {
       c->tail_nchunk = (int)std::min<int64_t>((E + cm - 1) / cm, 65);
       c->tail_chunk = (int)((std::min(cm, (E + c->tail_nchunk - 1) / c->tail_nchunk) + 3) & ~3);
       // a bucket's blocks: all full but its last one
@@ -768,16 +784,16 @@ void tt_pass_plan(tt_ctx* c) {
   c->head_sorted = c->pass_head && c->N / e2 <= HEAD_PLAN_MAX;
 }
 
-unsigned tt_pass_mask(const tt_ctx* c) {
+unsigned tt_pass_mask(const tt_ctx* c, const void* A) {
   unsigned m = c->pass_head ? 3u : 0u;
-  for (int s = 0; s < c->tail_modes; ++s) m |= 1u << (c->d - 1 - s);
+  for (int s = 0; s < c->tail_modes && tail_takes(c, A); ++s) m |= 1u << (c->d - 1 - s);
   return m;
 }
 
 // modes whose fibre plan an all-modes data sketch reads: every mode without a pass, and mode 1 where
 // the head pass takes its slabs from it
-unsigned tt_pass_plans(const tt_ctx* c) {
-  return (((1u << c->d) - 1u) & ~tt_pass_mask(c)) | (c->pass_head && !c->head_sorted ? 2u : 0u);
+unsigned tt_pass_plans(const tt_ctx* c, const void* A) {
+  return (((1u << c->d) - 1u) & ~tt_pass_mask(c, A)) | (c->pass_head && !c->head_sorted ? 2u : 0u);
 }
 
 int tt_launch_pass_plans(tt_ctx* c) {
@@ -887,8 +903,8 @@ int tt_launch_tail_pass(tt_ctx* c, const void* A, const float* scales, float* Ys
 // The data sketches of all modes on c->stream: the passes, then one launch per remaining mode; ev[k]
 // (when given) is recorded after Y_k.
 int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev) {
-  TT_TRY(tt_ensure_plans(c, tt_pass_plans(c), true));
-  const unsigned mask = tt_pass_mask(c);
+  TT_TRY(tt_ensure_plans(c, tt_pass_plans(c, A), true));
+  const unsigned mask = tt_pass_mask(c, A);
   const int64_t bytes = c->N * tt_elem_bytes(c->dtype) + (c->dtype == TT_FP8E4M3 ? 4 * c->n[0] : 0);
   auto mark = [&](int k) -> int {  // Y_k is done
     if (ev) TT_CUDA(c, cudaEventRecord(ev[k], c->stream));
@@ -914,7 +930,7 @@ int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* c
       TT_TRY(mark(k));
     }
   const int l = c->d - 1;
-  if (c->pass_tail)
+  if (tail_takes(c, A))
     TT_TRY(timed(c->d - c->tail_modes, l, [&] { return tt_launch_tail_pass(c, A, scales, Y[l - 1], Y[l]); }));
   return TT_OK;
 }

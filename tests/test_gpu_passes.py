@@ -81,6 +81,13 @@ def test_fp8_row_scales_beside_the_tail_chunk(n0):
     _check((n0, 3, 4), 8192, "fp8", columns=3, rank=1)
 
 
+@pytest.mark.parametrize("offset", [0, 4, 1])
+def test_fp8_chunks_above_10240_entries(offset):
+    """Four FP8 entries to a load reach 20,480 entries per chunk: slabs of two such chunks, and a base off
+    the 4-byte grid, which goes one launch per mode."""
+    _check((40, 30, 20, 5, 3), 2048, "fp8", offset, columns=3)
+
+
 def test_more_slabs_than_one_cta_sorts():
     """33,800 slabs of 512 entries: the head pass takes them from mode 1's grid-wide plan."""
     _check((32, 16, 130, 260), 1024, "f32", columns=3)

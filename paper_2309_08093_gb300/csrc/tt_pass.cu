@@ -647,18 +647,19 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
 }
 
 // CTAs of a pass with per_sm resident on an SM: one wave.
-// - Beside the chain of a single-tensor sweep it covers four fifths of the SMs: the passes' CTAs hold
-//   an SM's registers until they end, and the chain's kernels run on the others (100^4 FP32: 732 us
-//   per monitored sweep with a whole wave, 674, 639 and 640 us with 136, 120 and 104 tail CTAs, 626
-//   with the head pass cut the same way).
-// - In a batch at most one CTA per half an item's bytes, so that small tensors' passes run side by
-//   side (256 tensors: 14.50 ms per batched sweep without the bound, 13.83 ms with it; 32 tensors:
-//   2.50 ms; 2.81, 2.41, 2.40 and 2.46 ms at 1 MB, 512, 256 and 128 KB per CTA).
+// - In a sweep it covers four fifths of the SMs: the passes' CTAs hold an SM's registers until they
+//   end, and the chain's kernels (in a batch, also the other tensors') run on the rest. 100^4 FP32:
+//   732 us per monitored sweep with a whole wave, 674, 639 and 640 us with 136, 120 and 104 tail CTAs,
+//   626 with the head pass cut the same way. Batch of 4 tensors, the largest 66 M entries: 465 us
+//   with a whole wave, 423 with four fifths.
+// - In a batch also at most one CTA per 64 KB of A, so that small tensors' passes run side by side. 28
+//   batches of 4 to 32 tensors, mean speed against one launch per mode: 1.10 with 512 KB, 1.28 (256),
+//   1.32 (128), 1.33 (64 and 32); 256 tensors 1.24 from 256 KB down. Longer shares leave a tensor's
+//   chain waiting for a few CTAs (6 tensors of 5.5 M entries in all: 705 us, 310 with 64 KB).
 int64_t pass_ctas(const tt_ctx* c, int per_sm) {
   const int64_t sms = tt_sm_count();
-  const int64_t covered = c->in_sweep && !c->capture_mode ? sms * 4 / 5 : sms;
-  int64_t ctas = std::max<int64_t>(1, covered) * std::max(1, per_sm);
-  if (c->item_bytes > 0) ctas = std::min(ctas, 2 * c->N * tt_elem_bytes(c->dtype) / c->item_bytes);
+  int64_t ctas = std::max<int64_t>(1, c->in_sweep ? sms * 4 / 5 : sms) * std::max(1, per_sm);
+  if (c->item_bytes > 0) ctas = std::min(ctas, 16 * c->N * tt_elem_bytes(c->dtype) / c->item_bytes);
   return std::max<int64_t>(1, ctas);
 }
 

@@ -294,7 +294,10 @@ __global__ void __launch_bounds__(256) k_head_out(float* __restrict__ Y0r, float
 // CTA nchunk (when R > 0): the slabs of the head pass sorted by c, the hash of the modes 2 .. d-1
 // (plan word: fibre index of the slab | sign << 31). One CTA sorts up to 2^15 slabs; with more the
 // grid-wide plan of mode 1 (tt_context.cu) is used.
-// Both are counting sorts: counts in shared memory, a scan over the J buckets, placement.
+// Both are counting sorts: counts in shared memory, a scan over the J buckets, placement in shared
+// memory and coalesced stores. Bound by the latency of one CTA: with the tables' draw 14 us of a
+// fresh-draw call at 101 x 84 x 93 x 100 (22 us when every entry was hashed twice and stored where it
+// belongs), 15 us at 100^4 (30).
 struct PassPlanArgs {
   const int32_t* h;
   const int8_t* v;
@@ -304,6 +307,7 @@ struct PassPlanArgs {
   uint16_t* list;    // 4 * blocks numbers per chunk
   uint32_t* bucket;  // J words per chunk
   uint32_t* sign;    // (chunk + 31) / 32 words per chunk
+  int nkeys;         // entries or slabs that a CTA sorts, at most
   int64_t R;         // slabs of the head pass (0: not planned here)
   uint32_t* plan;
   int32_t* key;
@@ -312,6 +316,8 @@ constexpr int64_t HEAD_PLAN_MAX = 1 << 15;
 
 __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
   extern __shared__ int psm[];  // J counts, then cursors
+  uint16_t* keys = reinterpret_cast<uint16_t*>(psm + ((a.J + 1) & ~1));  // buckets (J <= 8192), sign in bit 15
+  uint16_t* ord = keys + a.nkeys;  // the sorted numbers, on their way to coalesced stores
   __shared__ int wsum[32];
   const int t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5;
   const bool slabs = (int)blockIdx.x == a.nchunk;
@@ -320,25 +326,36 @@ __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
   const int ne = slabs ? (int)a.R : (int)min((int64_t)a.chunk, a.E - e0);
   for (int b = t; b < a.J; b += T) psm[b] = 0;
   __syncthreads();
-  auto decode = [&](int i, int& neg) {
-    uint32_t rem = (uint32_t)(e0 + i);
-    int b = 0;
-    neg = 0;
-    for (int s = m0; s < m1; ++s) {
-      const uint32_t n = (uint32_t)a.n[s], q = rem / n, x = rem - q * n;
-      rem = q;
-      b = tt_modj(b + __ldg(a.h + a.noff[s] + x), a.J);
-      neg ^= __ldg(a.v + a.noff[s] + x) < 0;
-    }
-    return b;
-  };
   uint32_t* sign = a.sign + (int64_t)blockIdx.x * ((a.chunk + 31) / 32);
-  for (int i0 = 0; i0 < ne; i0 += T) {
-    const int i = i0 + t;
-    int neg = 0;
-    if (i < ne) atomicAdd(psm + decode(i, neg), 1);
-    const uint32_t w = __ballot_sync(0xffffffffu, neg);
-    if (!slabs && lane == 0 && i < ne) sign[i >> 5] = w;
+  constexpr int U = 4;  // entries whose table lookups are in flight together
+  for (int i0 = t; i0 - t < ne; i0 += U * T) {
+    uint32_t rem[U];
+    int key[U], neg[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      rem[u] = (uint32_t)(e0 + min(i0 + u * T, ne - 1));
+      key[u] = neg[u] = 0;
+    }
+    for (int s = m0; s < m1; ++s) {
+      const uint32_t n = (uint32_t)a.n[s];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t q = rem[u] / n, x = rem[u] - q * n;
+        rem[u] = q;
+        key[u] = tt_modj(key[u] + __ldg(a.h + a.noff[s] + x), a.J);
+        neg[u] ^= __ldg(a.v + a.noff[s] + x) < 0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * T;
+      const uint32_t w = __ballot_sync(0xffffffffu, neg[u] && i < ne);
+      if (i < ne) {
+        atomicAdd(psm + key[u], 1);
+        keys[i] = (uint16_t)(key[u] | neg[u] << 15);
+        if (!slabs && lane == 0) sign[i >> 5] = w;
+      }
+    }
   }
   __syncthreads();
   // exclusive scan of the J counts (block counts for a pattern): each thread a run of buckets
@@ -363,7 +380,6 @@ __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
   __syncthreads();
   int at = (warp ? wsum[warp - 1] : 0) + inc - sum;
   uint32_t* bucket = a.bucket + (int64_t)blockIdx.x * a.J;
-  uint16_t* list = a.list + (int64_t)blockIdx.x * a.blocks * 4;
   for (int b = lo; b < hi; ++b) {
     const int cnt = psm[b];
     if (slabs) {
@@ -372,21 +388,23 @@ __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
     } else {
       const int nb = (cnt + 3) >> 2;
       bucket[b] = (uint32_t)at | (uint32_t)nb << 16;
-      for (int i = cnt; i < 4 * nb; ++i) list[4 * at + i] = (uint16_t)a.chunk;
+      for (int i = cnt; i < 4 * nb; ++i) ord[4 * at + i] = (uint16_t)a.chunk;
       psm[b] = 4 * at;
       at += nb;
     }
   }
   __syncthreads();
-  for (int i = t; i < ne; i += T) {
-    int neg;
-    const int key = decode(i, neg), pos = atomicAdd(psm + key, 1);
-    if (slabs) {
-      a.plan[pos] = (uint32_t)((int64_t)i * a.n[1]) | (uint32_t)neg << 31;
-      a.key[pos] = key;
-    } else {
-      list[pos] = (uint16_t)i;
+  for (int i = t; i < ne; i += T) ord[atomicAdd(psm + (keys[i] & 0x7FFF), 1)] = (uint16_t)i;
+  __syncthreads();
+  if (slabs) {
+    for (int p = t; p < ne; p += T) {
+      const int i = ord[p], key = keys[i];
+      a.plan[p] = (uint32_t)((int64_t)i * a.n[1]) | (uint32_t)(key >> 15) << 31;
+      a.key[p] = key & 0x7FFF;
     }
+  } else {  // (wsum[31]: blocks of all buckets)
+    uint2* list = reinterpret_cast<uint2*>(a.list) + (int64_t)blockIdx.x * a.blocks;
+    for (int p = t; p < wsum[31]; p += T) list[p] = reinterpret_cast<const uint2*>(ord)[p];
   }
 }
 
@@ -820,7 +838,12 @@ int tt_launch_pass_plans(tt_ctx* c) {
   p.key = c->d_rkey;
   const int ctas = p.nchunk + (c->head_sorted ? 1 : 0);
   if (ctas == 0) return TT_OK;
-  k_pass_plans<<<ctas, 1024, sizeof(int) * (size_t)c->J, c->stream>>>(p);
+  // at most 4 J (J <= 8192) + 2 * 2^15 + 8 blocks (chunk / 4 + J): 202 KB
+  p.nkeys = (int)((std::max<int64_t>(p.nchunk ? p.chunk : 0, p.R) + 3) & ~3);
+  const size_t smem = sizeof(int) * (size_t)((c->J + 1) & ~1) +
+                      sizeof(uint16_t) * (p.nkeys + std::max<size_t>(p.nchunk ? 4 * (size_t)p.blocks : 0, p.R));
+  TT_CUDA(c, cudaFuncSetAttribute(k_pass_plans, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_pass_plans<<<ctas, 1024, smem, c->stream>>>(p);
   TT_LAUNCH(c, "k_pass_plans");
   return TT_OK;
 }

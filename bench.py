@@ -26,9 +26,9 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "ALS sweeps/s + unfold-sketch HBM GB/s at equal rel. error vs plain FP32 GPU"
-# DRAM bytes (read + write) per data-sketch launch from an ncu capture of the current kernels,
-# per (workload, storage); the roofline reports null for anything not captured.
-UNFOLD_TRAFFIC = {("order4-100-r10", "f32"): 428.65e6}
+# DRAM bytes (read + write) per data sketch (two modes share one read of the tensor) from an ncu
+# capture of the current kernels, per (workload, storage); the roofline reports null for anything not captured.
+UNFOLD_TRAFFIC = {("order4-100-r10", "f32"): 204.8e6}
 UNIT = "sweeps/s"
 DEFAULT_WORKLOAD = "order4-100-r10"
 
@@ -388,7 +388,7 @@ def batched_pattern(dev, nsweeps=10, count=256):
         c.close()
     esz = {"f32": 4, "bf16": 2}
     tensor_bytes = sum(int(a.numel()) * esz[sp["dtype"]] for a, sp in zip(As, specs))
-    unfold_bytes = sum(int(a.numel()) * esz[sp["dtype"]] * len(sp["dims"]) for a, sp in zip(As, specs))
+    unfold_bytes = 2 * tensor_bytes  # the passes read a tensor of order 3 or 4 twice
     sweep_s = ms / 1e3 / nsweeps
     errs_sorted = sorted(errs)
     return {"tensors": count, "tensor_gb": tensor_bytes / 1e9, "sweeps": nsweeps,
@@ -403,7 +403,7 @@ def batched_pattern(dev, nsweeps=10, count=256):
                            "note": f"TT_FLAG_FIXED_SKETCH on every tensor; one call of {nsweeps} sweeps: the first "
                                    "computes the data sketches, the others reuse them"},
             "note": "noise 1e-3 (the floor); sweeps timed with CUDA events around one tt_batch_sweep call "
-                    "(graph replays); unfold GB/s = tensor bytes x order / sweep time, everything else in "
+                    "(graph replays); unfold GB/s = two reads of every tensor / sweep time, everything else in "
                     "the sweep included"}
 
 
@@ -1000,18 +1000,19 @@ def main():
                 "scaling": "weak", "vs_baseline": None, "dtype": storage, "data": "synthetic",
                 "config": workload_config(w, storage),
                 "rel_error_after": err,
-                "roofline": {"kernel": "data sketch (k_unfold_gather mode 0 + k_unfold_cols modes >= 1)",
+                "roofline": {"kernel": "data sketch (k_head_pass modes 0 and 1, k_tail_pass the last two, k_unfold_cols between)",
                              "bound": "hbm",
                              "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                              "peak_kind": peak_kind,
                              "traffic": UNFOLD_TRAFFIC.get((args.workload, storage)),
-                             "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum per launch, mean over the "
-                                             "four modes of one sweep (in-sweep launch shapes), from one ncu capture of "
-                                             "these kernel versions; null for workloads not captured",
+                             "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum per data sketch, mean over the "
+                                             "four modes (two per read of the tensor), from one ncu capture of these "
+                                             "kernel versions; null for workloads not captured",
                              "bytes_per_launch": bytes_per_launch, "avg_launch_ms": unfold_avg_ms,
                              "per_mode_gbs": mode_gbs,
                              "share_of_step": prof["unfold_ms"] / ms,
-                             "note": "CUDA events around every data-sketch launch in the timed region; the sweep "
+                             "note": "CUDA events around every data-sketch launch in the timed region (a launch that gives two "
+                                     "modes counts as two, half its time and bytes each); the sweep "
                                      "runs these kernels on a side stream concurrently with the chain kernels, so "
                                      "their durations include that sharing (see roofline_isolated)"},
                 "roofline_isolated": iso,

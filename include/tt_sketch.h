@@ -361,8 +361,9 @@ int tt_batch_rel_error(tt_batch* b, const void* const* A_dev, const float* const
 /* Per-context counters for measurement (not part of the method). */
 typedef struct {
   double unfold_ms;          /* summed device time of the unfold-sketch kernels (CUDA events) */
-  int64_t unfold_launches;   /* number of unfold-sketch kernel launches timed */
-  int64_t unfold_bytes;      /* algorithmic bytes those launches read: entries x storage size */
+  int64_t unfold_launches;   /* number of data sketches timed: a read of A that gives the sketches of
+                                two modes counts as two, and its time is shared between them */
+  int64_t unfold_bytes;      /* algorithmic bytes read for them: entries x storage size per read of A */
   int64_t kernel_launches;   /* every kernel this library launched since the reset */
   double mode_ms[8];         /* unfold device time per mode */
   int64_t mode_launches[8];

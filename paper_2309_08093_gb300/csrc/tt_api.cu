@@ -333,7 +333,7 @@ int tt_elem_bytes(int dtype) {
 // ---------------------------------------------------------------------------------------------
 // measurement counters
 
-int tt_prof_begin(tt_ctx* c, int k) {
+int tt_prof_begin(tt_ctx* c, int k0, int k1) {
   if (!c->profiling) return TT_OK;
   while ((int)c->ev_pool.size() < c->ev_used + 2) {
     cudaEvent_t e;
@@ -341,7 +341,7 @@ int tt_prof_begin(tt_ctx* c, int k) {
     c->ev_pool.push_back(e);
   }
   TT_CUDA(c, cudaEventRecord(c->ev_pool[c->ev_used], c->stream));
-  c->ev_mode.push_back(k);
+  c->ev_mode.push_back({k0, k1});
   c->ev_used += 1;
   return TT_OK;
 }
@@ -350,7 +350,7 @@ int tt_prof_end(tt_ctx* c) {
   if (!c->profiling) return TT_OK;
   TT_CUDA(c, cudaEventRecord(c->ev_pool[c->ev_used], c->stream));
   c->ev_used += 1;
-  // algorithmic bytes of one data-sketch launch: every entry once, plus the FP8 slice scales
+  // algorithmic bytes of one read of A: every entry once, plus the FP8 slice scales
   c->prof_bytes += (int64_t)c->N * tt_elem_bytes(c->dtype) + (c->dtype == TT_FP8E4M3 ? 4 * c->n[0] : 0);
   return TT_OK;
 }
@@ -375,11 +375,11 @@ extern "C" int tt_profile_read(tt_ctx* c, tt_profile* out) {
   for (int i = 0; i + 1 < c->ev_used; i += 2) {
     float ms = 0.f;
     TT_CUDA(c, cudaEventElapsedTime(&ms, c->ev_pool[i], c->ev_pool[i + 1]));
-    int k = c->ev_mode[i / 2];
+    const auto [k0, k1] = c->ev_mode[i / 2];
     out->unfold_ms += ms;
-    out->unfold_launches += 1;
-    if (k >= 0 && k < 8) {
-      out->mode_ms[k] += ms;
+    for (int k = k0; k <= k1; ++k) {  // a pass: its modes share its time
+      out->unfold_launches += 1;
+      out->mode_ms[k] += ms / (k1 - k0 + 1);
       out->mode_launches[k] += 1;
     }
   }

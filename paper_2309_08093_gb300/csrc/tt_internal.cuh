@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/tt_sketch.h"
@@ -202,7 +203,7 @@ struct tt_ctx {
   int64_t launches = 0;
   bool profiling = false;
   std::vector<cudaEvent_t> ev_pool;
-  std::vector<int> ev_mode;   // mode of each recorded pair (pairs at 2i, 2i+1)
+  std::vector<std::pair<int, int>> ev_mode;  // first and last mode of each recorded pair (at 2i, 2i+1)
   int ev_used = 0;            // events in use
   int64_t prof_bytes = 0;
 
@@ -367,7 +368,7 @@ int tt_check_data(tt_ctx* c, const void* A, const float* scales);
   } while (0)
 int tt_one_sweep(tt_ctx* c, const void* A, const float* scales, float* const* cores, uint64_t sweep,
                  double* change_slots, float* const* Ygiven = nullptr);
-int tt_prof_begin(tt_ctx* c, int k);   // record a start event when profiling (returns TT_OK)
+int tt_prof_begin(tt_ctx* c, int k0, int k1);  // record a start event when profiling (returns TT_OK)
 int tt_prof_end(tt_ctx* c);
 int tt_elem_bytes(int dtype);
 // number of SMs of the current device (queried once per device; 152 if the query fails)

@@ -448,7 +448,7 @@ __device__ __forceinline__ void add2(unsigned long long& q, unsigned long long x
 // registers while i_s advances, and adds its q to Y_s with atomics that are contiguous across a warp.
 // The next unit's slabs are loaded into registers meanwhile. The signs go on when a slab is staged.
 // Bound: instruction issue (61% active; 115 M warp instructions) and the random shared-memory loads
-// (150 k of 331 k cycles). 100^4 FP32: 160 us for both modes at J = 4096, 134 us at J = 1024 (one
+// (150 k of 331 k cycles). 100^4 FP32: 160 us for both modes at J = 4096, 127 us at J = 1024 (one
 // launch per mode: 206 and 172 us).
 template <int DT, int V, int EPW, int RPT>
 __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
@@ -929,21 +929,15 @@ int tt_launch_tail_pass(tt_ctx* c, const void* A, const float* scales, float* Ys
 int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev) {
   TT_TRY(tt_ensure_plans(c, tt_pass_plans(c, A), true));
   const unsigned mask = tt_pass_mask(c, A);
-  const int64_t bytes = c->N * tt_elem_bytes(c->dtype) + (c->dtype == TT_FP8E4M3 ? 4 * c->n[0] : 0);
   auto mark = [&](int k) -> int {  // Y_k is done
     if (ev) TT_CUDA(c, cudaEventRecord(ev[k], c->stream));
     return TT_OK;
   };
-  // a pass is timed as its first mode, its other modes as empty intervals (its bytes count once)
+  // a pass is timed as one read of A that its modes share
   auto timed = [&](int k0, int k1, auto&& pass) -> int {
-    TT_TRY(tt_prof_begin(c, k0));
+    TT_TRY(tt_prof_begin(c, k0, k1));
     TT_TRY(pass());
     TT_TRY(tt_prof_end(c));
-    for (int k = k0 + 1; k <= k1; ++k) {
-      TT_TRY(tt_prof_begin(c, k));
-      TT_TRY(tt_prof_end(c));
-      if (c->profiling) c->prof_bytes -= bytes;
-    }
     for (int k = k0; k <= k1; ++k) TT_TRY(mark(k));
     return TT_OK;
   };

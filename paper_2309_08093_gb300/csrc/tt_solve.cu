@@ -11,7 +11,8 @@
 //   k_lq_right    : the same on (G_k^R)^T: G_k^R <- Q^T, G_{k-1}^L <- G_{k-1}^L R^T
 //   k_slab_u, k_rint, k_rel_error_stream : ||A - [[G]]||_F^2 and ||A||_F^2: right interfaces of
 //                   all mode-0 fibres, then one pass over A in memory order (bulk copies)
-//   k_rel_error   : the same for other shapes (n_0 % 4 != 0 or n_0 > 1024), slab by slab
+//   k_rel_error   : the same for other shapes (n_0 % 4 != 0 or n_0 > 1024) and for tensors off the
+//                   16-byte grid, slab by slab
 #include <stdio.h>
 
 #include <algorithm>

@@ -1,4 +1,7 @@
 // Part (a): Y_k = S A_(k)^T, the TensorSketch of every mode-k unfolding (Alg. 1, Sec. 3).
+// One launch per mode. A call for all modes takes modes 0 and 1 and the last two from one read of A each
+// where the shape allows (tt_pass.cu); the kernels here take single modes, what the passes leave out and
+// the shapes and options without them.
 //
 // Y_k[b, i_k] = sum over entries with that i_k of prod_{s!=k} v_s(i_s) * A(i), restricted to
 // (sum_{s!=k} h_s(i_s)) mod J = b  (Eqs. (eqn_h), (eqn_v)).
@@ -330,7 +333,7 @@ int tt_launch_unfold(tt_ctx* c, const void* A, const float* scales, int k, float
 }
 
 int tt_launch_unfold_planned(tt_ctx* c, const void* A, const float* scales, int k, float* Y) {
-  int rc = tt_prof_begin(c, k);
+  int rc = tt_prof_begin(c, k, k);
   if (rc) return rc;
   switch (c->dtype) {
     case TT_F64: rc = unfold_dt<TT_F64>(c, A, scales, k, Y); break;

@@ -289,7 +289,9 @@ __global__ void __launch_bounds__(256) k_head_out(float* __restrict__ Y0r, float
 // CTA b < nchunk: the head's pattern of the tail pass, the same for every slab. The entries of a
 // slab, cut into chunks of `chunk` entries, are listed by bucket (sum of the head modes' hashes mod
 // J) within each chunk, in blocks of four 16-bit entry numbers; a bucket's last block is filled up
-// with number `chunk`, an entry that is staged as zero. Bucket word: first block | blocks << 16.
+// with a number from `chunk` on, an entry that is staged as zero (FP8: there are n_0 of them, and the
+// one of a row that the bucket holds is taken, so that no other row's scale, which may be infinite,
+// enters the sum). Bucket word: first block | blocks << 16.
 // Sign word: the signs (product of the head modes' v) of 32 entries.
 // CTA nchunk (when R > 0): the slabs of the head pass sorted by c, the hash of the modes 2 .. d-1
 // (plan word: fibre index of the slab | sign << 31). One CTA sorts up to 2^15 slabs; with more the
@@ -308,6 +310,7 @@ struct PassPlanArgs {
   uint32_t* bucket;  // J words per chunk
   uint32_t* sign;    // (chunk + 31) / 32 words per chunk
   int nkeys;         // entries or slabs that a CTA sorts, at most
+  int zeros;         // zero entries behind a staged chunk: a row each (FP8) or one
   int64_t R;         // slabs of the head pass (0: not planned here)
   uint32_t* plan;
   int32_t* key;
@@ -388,7 +391,6 @@ __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
     } else {
       const int nb = (cnt + 3) >> 2;
       bucket[b] = (uint32_t)at | (uint32_t)nb << 16;
-      for (int i = cnt; i < 4 * nb; ++i) ord[4 * at + i] = (uint16_t)a.chunk;
       psm[b] = 4 * at;
       at += nb;
     }
@@ -396,6 +398,14 @@ __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
   __syncthreads();
   for (int i = t; i < ne; i += T) ord[atomicAdd(psm + (keys[i] & 0x7FFF), 1)] = (uint16_t)i;
   __syncthreads();
+  if (!slabs) {  // fill up last blocks (they start at multiples of 4)
+    for (int b = lo; b < hi; ++b) {
+      int p = psm[b];
+      if (p & 3)
+        for (const int e = ord[p - 1], m = a.zeros, z = a.chunk + ((e - a.chunk) % m + m) % m; p & 3; ++p) ord[p] = (uint16_t)z;
+    }
+    __syncthreads();
+  }
   if (slabs) {
     for (int p = t; p < ne; p += T) {
       const int i = ord[p], key = keys[i];
@@ -456,15 +466,16 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
   constexpr int EB = Sh::EB, JJ = Sh::JJ, ENT = Sh::ENT, T = TAIL_T;
   using Word = typename std::conditional<EB == 8, double, uint32_t>::type;
   extern __shared__ __align__(16) unsigned char tsm[];
-  unsigned char* buf = tsm;                                                                  // chunk + 1 entries
-  uint2* sl = reinterpret_cast<uint2*>(buf + (((size_t)(a.chunk + 1) * ENT + 15) & ~(size_t)15));  // blocks
+  const int zeros = DT == TT_FP8E4M3 ? a.n0 : 1;
+  unsigned char* buf = tsm;  // chunk + zeros entries
+  uint2* sl = reinterpret_cast<uint2*>(buf + (((size_t)(a.chunk + zeros) * ENT + 15) & ~(size_t)15));  // blocks
   uint32_t* sb = reinterpret_cast<uint32_t*>(sl + a.blocks);                                 // J
   float* ssc = reinterpret_cast<float*>(sb + a.J);                                           // n0 FP8 scales
   const int t = threadIdx.x, J = a.J, parts = a.parts;
   const int part = t & (parts - 1), row0 = t / parts, rstep = T / parts;
   if (DT == TT_FP8E4M3)
     for (int i = t; i < a.n0; i += T) ssc[i] = __ldg(a.scales + i);
-  if (t < ENT) buf[(size_t)a.chunk * ENT + t] = 0;
+  for (int i = t; i < zeros * ENT; i += T) buf[(size_t)a.chunk * ENT + i] = 0;
   const int64_t u0 = a.units * blockIdx.x / gridDim.x, u1 = a.units * (blockIdx.x + 1) / gridDim.x;
   if (u0 >= u1) return;
   int is = (int)(u0 % a.ns), gl = (int)((u0 / a.ns) % a.ngl), ch = (int)(u0 / a.ns / a.ngl);
@@ -681,9 +692,9 @@ int64_t pass_ctas(const tt_ctx* c, int per_sm) {
   return std::max<int64_t>(1, ctas);
 }
 
-// shared memory of k_tail_pass: chunk + 1 staged entries, lists, buckets, row scales
+// shared memory of k_tail_pass: a staged chunk and its zero entries, lists, buckets, row scales
 size_t tail_smem(int64_t chunk, int64_t blocks, int64_t J, int64_t entry_bytes, int64_t nscales) {
-  return ((size_t)((chunk + 1) * entry_bytes + 15) & ~(size_t)15) + (size_t)(8 * blocks + 4 * J + 4 * nscales);
+  return ((size_t)((chunk + std::max<int64_t>(nscales, 1)) * entry_bytes + 15) & ~(size_t)15) + (size_t)(8 * blocks + 4 * J + 4 * nscales);
 }
 
 template <int DT, int V, int EPW>
@@ -829,6 +840,7 @@ int tt_launch_pass_plans(tt_ctx* c) {
   p.chunk = c->tail_chunk;
   p.nchunk = c->pass_tail ? c->tail_nchunk : 0;
   p.blocks = c->tail_blocks;
+  p.zeros = c->dtype == TT_FP8E4M3 ? (int)c->n[0] : 1;
   p.E = c->stride[p.nh];
   p.list = c->d_tlist;
   p.bucket = c->d_tbucket;

@@ -75,9 +75,9 @@ def test_tensor_off_the_16_byte_grid(dtype, offset):
     _check((32, 24, 7, 5), 256, dtype, offset)
 
 
-@pytest.mark.parametrize("n0", [6000, 24000, 40000])
+@pytest.mark.parametrize("n0", [6000, 14000, 24000, 40000])
 def test_fp8_row_scales_beside_the_tail_chunk(n0):
-    """A scale per row of A in shared memory: whole chunks, shorter ones, and no tail pass."""
+    """A scale and a zero entry per row of A in shared memory: whole chunks, shorter ones, no tail pass."""
     _check((n0, 3, 4), 8192, "fp8", columns=3, rank=1)
 
 
@@ -86,6 +86,26 @@ def test_fp8_chunks_above_10240_entries(offset):
     """Four FP8 entries to a load reach 20,480 entries per chunk: slabs of two such chunks, and a base off
     the 4-byte grid, which goes one launch per mode."""
     _check((40, 30, 20, 5, 3), 2048, "fp8", offset, columns=3)
+
+
+@pytest.mark.parametrize("row", [0, 13, 31])
+def test_an_infinite_row_scale_stays_in_its_buckets(row):
+    """FP8 with one infinite scale: a sum is not finite exactly where an entry of that row falls."""
+    dims, J, seed = (32, 24, 7, 5), 4096, 977
+    flat, scales, _ = synth.quantize(synth.random_tensor(dims, 31), "fp8")
+    scales = scales.copy()
+    scales[row] = np.inf
+    ctx = lib.Context(dims, [1, 2, 2, 2, 1], J, 1e-3, seed, "fp8")
+    Y = [torch.empty(n, J, device="cuda") for n in dims]
+    ctx.tt_sketch_unfold(lib.device_tensor(flat, "fp8"), -1, 4, Y, torch.from_numpy(scales).cuda())
+    hs, vs = O.draw_sketch(seed, 4, dims, J)
+    hit = np.zeros(dims)
+    hit[row] = 1.0
+    ones = [np.ones_like(v) for v in vs]
+    for k, n in enumerate(dims):
+        bad = np.stack([O.sketch_unfolding_column(hit, hs, ones, J, k, i) for i in range(n)]) > 0
+        assert np.array_equal(~np.isfinite(Y[k].cpu().numpy()), bad), k
+    ctx.close()
 
 
 def test_more_slabs_than_one_cta_sorts():

@@ -699,6 +699,7 @@ static void tt_workspace_each(tt_ctx* c, F&& A) {
     A((void**)&c->d_tbucket, b);
     A((void**)&c->spare.tlist, e);
     A((void**)&c->spare.tbucket, b);
+    if (tt_tail_copies(c) > 0) A((void**)&c->d_ysl, sizeof(float) * (size_t)tt_tail_copies(c));
   }
   if (c->det) {
     A((void**)&c->d_det_misc, sizeof(int) * 4);
@@ -881,6 +882,7 @@ extern "C" int tt_sketch_init(tt_ctx** out, const tt_params* p, void* stream) {
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
   if (e == cudaSuccess && c->d_y01)
     e = cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)c->J * (c->p0 + c->p1), c->stream);
+  if (e == cudaSuccess && c->d_ysl) e = cudaMemsetAsync(c->d_ysl, 0, sizeof(float) * (size_t)tt_tail_copies(c), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
     free_all(c);

@@ -136,6 +136,7 @@ struct tt_ctx {
   int tail_modes = 0;
   int tail_chunk = 0, tail_nchunk = 0;  // entries per chunk of a tail-pass slab, chunks
   int tail_blocks = 0;                  // list blocks per chunk, at most
+  int tail_cs = 1, tail_cl = 1;         // copies of Y_s and Y_l that the tail pass adds into (powers of two)
   int p0 = 0, p1 = 0;                   // row lengths of the head pass's accumulators (n_0, n_1 up to 4s)
   bool head_sorted = false;             // the head pass's slabs are sorted by k_pass_plans (else mode 1's plan)
   uint32_t* d_hplan = nullptr;          // head pass: slabs by c (when head_sorted)
@@ -145,6 +146,8 @@ struct tt_ctx {
   bool pass_valid = false;              // d_hplan, d_tlist, d_tbucket are those of the current draw
   float* d_y01 = nullptr;               // J x p0 then J x p1: Y_0 and Y_1 by rows (zero between head passes)
   bool y01_zero = true;                 // they are (false after a launch that failed in between)
+  float* d_ysl = nullptr;               // tail_cs copies of Y_s, then tail_cl of Y_l, those above one (zero likewise)
+  bool ysl_zero = true;
   TtDraw spare;                              // the next sweep's draw (see TtDraw)
   cudaEvent_t ev_spare = nullptr;            // end of the spare's build on `side`
   bool spare_pending = false;
@@ -315,6 +318,7 @@ int tt_launch_unfold_planned(tt_ctx* c, const void* A, const float* scales, int 
 // allows, tt_launch_unfold for the other modes; ev[k] (optional) is recorded after Y[k]
 int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev = nullptr);
 void tt_pass_plan(tt_ctx* c);                 // which modes the passes cover, from the shape
+int64_t tt_tail_copies(const tt_ctx* c);      // floats of d_ysl
 unsigned tt_pass_mask(const tt_ctx* c, const void* A);   // modes of A covered by the passes
 unsigned tt_pass_plans(const tt_ctx* c, const void* A);  // modes whose fibre plan tt_launch_unfold_all reads
 int tt_launch_pass_plans(tt_ctx* c);          // d_hplan, d_rkey, d_tlist, d_tbucket of the current draw

@@ -14,6 +14,7 @@
 //     Y_l[(c + h_s(i_s)) mod J, i_l] += v_s(i_s) q_t[c],   Y_s[(c + h_l(i_l)) mod J, i_s] += v_l(i_l) q_t[c],
 // again one read of A for both. The modes between (d >= 5) keep one launch each (tt_unfold.cu).
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "tt_unfold.cuh"
@@ -21,6 +22,33 @@
 namespace {
 
 __device__ __forceinline__ void red4(float* p, float4 v) { atomicAdd(reinterpret_cast<float4*>(p), v); }
+
+// Sum of the n values p[0], p[stride], ..., which are left zero: an unevaluated pair of floats (two-sums),
+// so that only its rounding to one float counts
+__device__ __forceinline__ float take_copies(float* p, int64_t stride, int n) {
+  float s = 0.f, e = 0.f;
+  for (int c = 0; c < n; c += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = c + u < n ? p[(c + u) * stride] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (c + u < n) p[(c + u) * stride] = 0.f;
+      const float t = s + v[u], b = t - s;
+      e += (s - (t - b)) + (v[u] - b);
+      s = t;
+    }
+  }
+  return isfinite(e) ? s + e : s;  // (an infinite sum has no error term)
+}
+
+// copies of an accumulator whose entries take `adds` FP32 adds one after the other: about sqrt(adds), a
+// power of two, so that the adds to a copy and the copies are two short sums
+int copies_of(double adds) {
+  int c = 1;
+  while (2.0 * c * c < adds && c < 64) c *= 2;  // nearest power of two on a logarithmic scale
+  return c;
+}
 
 // ---------------------------------------------------------------------------------------------
 // head pass
@@ -316,6 +344,7 @@ struct PassPlanArgs {
   int32_t* key;
 };
 constexpr int64_t HEAD_PLAN_MAX = 1 << 15;
+constexpr int64_t PASS_COPIES_MAX = 24 << 20;  // floats of a pass's accumulators (they are to stay in L2)
 
 __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
   extern __shared__ int psm[];  // J counts, then cursors
@@ -425,7 +454,8 @@ struct TailArgs {
   const uint32_t *bucket, *sign;
   const int32_t *hs, *hl;  // hashes and signs of the tail modes s (null: one tail mode) and l
   const int8_t *vs, *vl;
-  float *Ys, *Yl;  // J x n_s, J x n_l column-major, zeroed
+  float *Ys, *Yl;  // cs copies of J x n_s, cl copies of J x n_l, column-major, zeroed
+  int cs, cl;      // powers of two
   int64_t E;       // entries of a slab
   int J, n0, chunk, nchunk, blocks, ns, nl, ngl;  // ngl: groups of V indices i_l
   int parts;       // lanes that share a bucket's list (a power of two)
@@ -434,6 +464,9 @@ struct TailArgs {
 };
 
 constexpr int TAIL_T = 1024;
+// Slabs that Y_l's registers sum before they are added to a copy. FP8 launches of one mode add a row's
+// entries exactly before its scale rounds them, so their sums are the shortest to match.
+__host__ __device__ constexpr int tail_run(int dtype) { return dtype == TT_FP8E4M3 ? 4 : 8; }
 
 // What a thread stages per slab group: JJ loads of EPW entries from each of V slabs. An entry of the
 // staged chunk holds its V slabs' signed values side by side (V * SB bytes), so that one
@@ -455,11 +488,18 @@ __device__ __forceinline__ void add2(unsigned long long& q, unsigned long long x
 // One CTA of 1024 threads per SM; unit = (chunk, group of V indices i_l, i_s), consecutive units in one
 // CTA. Thread t owns bucket b of Y_l and so, per i_s, the head's bucket b - h_s(i_s): it sums that
 // bucket's list from the staged slabs (random 8-byte shared-memory loads), keeps Y_l's column sums in
-// registers while i_s advances, and adds its q to Y_s with atomics that are contiguous across a warp.
-// The next unit's slabs are loaded into registers meanwhile. The signs go on when a slab is staged.
+// registers while i_s advances (tail_run slabs at most), and adds its q to Y_s with atomics that are
+// contiguous across a warp. The next unit's slabs are loaded into registers meanwhile. The signs go on
+// when a slab is staged.
+// Accuracy: FP32 sums of n terms one after the other carry a rounding error that grows with sqrt(n), and
+// a bucket of Y_s takes up to n_l * nchunk of these adds, one of Y_l n_s * nchunk. They are cut in two
+// levels: units go to one of cs (cl) copies of Y_s (Y_l) in turn, and k_tail_out adds the copies up; the
+// lists are summed block by block where a bucket has several. Relative error of Y_s, one sum / in levels /
+// one launch per mode: 256 x 256 x 3 x 128 FP32 5.4e-7 / 1.1e-7 / 2.0e-7, 40^5 FP8 2.2e-7 / 7.3e-8 /
+// 7.8e-8, 100^4 FP32 1.8e-7 / 7.9e-8 / 9.5e-8.
 // Bound: instruction issue (61% active; 115 M warp instructions) and the random shared-memory loads
-// (150 k of 331 k cycles). 100^4 FP32: 160 us for both modes at J = 4096, 127 us at J = 1024 (one
-// launch per mode: 206 and 172 us).
+// (150 k of 331 k cycles). 100^4 FP32: 181 us for both modes at J = 4096 (160 us without the copies, one
+// launch per mode 206 us).
 template <int DT, int V, int EPW, int RPT>
 __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
   using Sh = TailShape<DT, V, EPW>;
@@ -566,15 +606,16 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
   for (int j = 0; j < RPT; ++j)
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[j][v] = 0.f;
-  auto flush = [&](int gl_) {  // the group's columns of Y_l
+  auto flush = [&](int gl_, int at) {  // the group's columns of Y_l, into copy `at` mod cl
     if (part == 0) {
+      float* yl = a.Yl + (int64_t)(at & (a.cl - 1)) * J * a.nl;
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         const int b = row0 + rstep * j;
         if (b < J) {
 #pragma unroll
           for (int v = 0; v < V; ++v)
-            if (V * gl_ + v < a.nl && acc[j][v] != 0.f) atomicAdd(a.Yl + (int64_t)J * (V * gl_ + v) + b, acc[j][v]);
+            if (V * gl_ + v < a.nl && acc[j][v] != 0.f) atomicAdd(yl + (int64_t)J * (V * gl_ + v) + b, acc[j][v]);
         }
       }
     }
@@ -619,7 +660,7 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
     if (a.hs) {
       hs = __ldg(a.hs + is);
       vs = __ldg(a.vs + is) < 0 ? -1.f : 1.f;
-      ys = a.Ys + (int64_t)J * is;
+      ys = a.Ys + (int64_t)J * (((ch * a.ngl + gl) & (a.cs - 1)) * a.ns + is);
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         const int il = min(V * gl + v, a.nl - 1);
@@ -643,19 +684,30 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
         unsigned long long qq = 0;
         for (int p = p0 + part; p < pe; p += parts) {
           const uint2 x = sl[p];
-          add2(qq, src[x.x & 0xFFFFu]);
-          add2(qq, src[x.x >> 16]);
-          add2(qq, src[x.y & 0xFFFFu]);
-          add2(qq, src[x.y >> 16]);
+          unsigned long long lo = src[x.x & 0xFFFFu], hi = src[x.y & 0xFFFFu];  // a block in pairs
+          add2(lo, src[x.x >> 16]);
+          add2(hi, src[x.y >> 16]);
+          add2(lo, hi);
+          add2(qq, lo);
         }
         q[0] = __uint_as_float((uint32_t)qq), q[1] = __uint_as_float((uint32_t)(qq >> 32));
       } else {
         for (int p = p0 + part; p < pe; p += parts) {
           const uint2 x = sl[p];
-          gather(x.x & 0xFFFFu, q);
-          gather(x.x >> 16, q);
-          gather(x.y & 0xFFFFu, q);
-          gather(x.y >> 16, q);
+          if constexpr (RPT <= 2) {  // buckets of several blocks: each block on its own
+            float qb[V] = {};
+            gather(x.x & 0xFFFFu, qb);
+            gather(x.x >> 16, qb);
+            gather(x.y & 0xFFFFu, qb);
+            gather(x.y >> 16, qb);
+#pragma unroll
+            for (int v = 0; v < V; ++v) q[v] += qb[v];
+          } else {
+            gather(x.x & 0xFFFFu, q);
+            gather(x.x >> 16, q);
+            gather(x.y & 0xFFFFu, q);
+            gather(x.y >> 16, q);
+          }
         }
       }
       if (parts > 1)
@@ -670,9 +722,24 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
           if (v < nv) atomicAdd(ys + tt_modj(c + hl[v], J), vl[v] * q[v]);
       }
     }
-    if (ngl != gl || nch != ch || u + 1 == u1) flush(gl);
+    constexpr int RUN = tail_run(DT);
+    if (ngl != gl || nch != ch || u + 1 == u1 || (is + 1) % RUN == 0) flush(gl, ch * ((a.ns + RUN - 1) / RUN) + is / RUN);
     is = nis, gl = ngl, ch = nch;
   }
+}
+
+// The copies of Y_s and of Y_l added up (and left zero for the next tail pass); bound by the L2 reads and
+// stores of the copies.
+struct TailOutArgs {
+  float* src[2];
+  float* dst[2];
+  int64_t n[2];  // entries of a copy
+  int copies[2];
+};
+__global__ void __launch_bounds__(256) k_tail_out(TailOutArgs a) {
+  for (int z = 0; z < 2; ++z)
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n[z]; i += (int64_t)gridDim.x * 256)
+      a.dst[z][i] = take_copies(a.src[z] + i, a.n[z], a.copies[z]);
 }
 
 // CTAs of a pass with per_sm resident on an SM: one wave.
@@ -809,9 +876,23 @@ void tt_pass_plan(tt_ctx* c) {
       fits = tail_smem(c->tail_chunk, c->tail_blocks, c->J, fp8 ? 4 : 8, fp8 ? c->n[0] : 0) <= 227 * 1024;
     }
     c->pass_tail = fits && E >= 512 && E * 8 >= c->J && c->tail_nchunk <= 64;
-    if (c->pass_tail) c->tail_modes = nt;
+    if (c->pass_tail) {
+      const double slabs = (double)c->tail_nchunk * c->n[c->d - 1];  // that a bucket of Y_s meets
+      c->tail_cs = nt == 2 ? copies_of((fp8 ? 2.0 : 1.0) * slabs * -std::expm1(-(double)c->tail_chunk / c->J)) : 1;
+      const int run = tail_run(c->dtype);
+      c->tail_cl = copies_of((fp8 ? 3.0 : 2.0) * c->tail_nchunk * (nt == 2 ? (c->n[c->d - 2] + run - 1) / run : 1));
+      c->tail_modes = nt;
+      if (tt_tail_copies(c) > PASS_COPIES_MAX) c->pass_tail = false, c->tail_modes = 0;
+    }
   }
   c->head_sorted = c->pass_head && c->N / e2 <= HEAD_PLAN_MAX;
+}
+
+int64_t tt_tail_copies(const tt_ctx* c) {
+  int64_t n = 0;
+  if (c->tail_cs > 1) n += c->tail_cs * c->J * c->n[c->d - 2];
+  if (c->tail_cl > 1) n += c->tail_cl * c->J * c->n[c->d - 1];
+  return n;
 }
 
 unsigned tt_pass_mask(const tt_ctx* c, const void* A) {
@@ -882,10 +963,11 @@ int tt_launch_head_pass(tt_ctx* c, const void* A, const float* scales, float* co
   a.nch = (a.n1 + a.G1 - 1) / a.G1;
   a.pitch = (a.n0 + 31) & ~31;
   a.inv_n0 = (uint32_t)((((uint64_t)1 << 32) + a.n0 - 1) / a.n0);
-  for (int z = 0; z < c->tail_modes; ++z) {
-    a.zero[z] = Y[c->d - 1 - z];
-    a.nzero[z] = (int64_t)c->J * c->n[c->d - 1 - z];
-  }
+  for (int z = 0; z < c->tail_modes; ++z)
+    if ((z == 0 ? c->tail_cl : c->tail_cs) == 1) {
+      a.zero[z] = Y[c->d - 1 - z];
+      a.nzero[z] = (int64_t)c->J * c->n[c->d - 1 - z];
+    }
   if (!c->y01_zero) TT_CUDA(c, cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)c->J * (c->p0 + c->p1), c->stream));
   c->y01_zero = false;
   switch (c->dtype) {
@@ -913,14 +995,22 @@ int tt_launch_tail_pass(tt_ctx* c, const void* A, const float* scales, float* Ys
   a.inv_n0 = (uint32_t)((((uint64_t)1 << 32) + c->n[0] - 1) / c->n[0]);
   a.hl = c->d_h + c->noff[l];
   a.vl = c->d_v + c->noff[l];
+  a.cs = c->tail_cs;
+  a.cl = c->tail_cl;
   if (c->tail_modes == 2) {
     a.hs = c->d_h + c->noff[s];
     a.vs = c->d_v + c->noff[s];
-    a.Ys = Ys;
+    a.Ys = a.cs > 1 ? c->d_ysl : Ys;
   }
-  a.Yl = Yl;
+  const int64_t ls = a.cs > 1 ? (int64_t)c->J * c->n[s] : 0, ll = (int64_t)c->J * c->n[l];  // a copy's entries
+  a.Yl = a.cl > 1 ? c->d_ysl + a.cs * ls : Yl;
   for (int k = l; k > l - c->tail_modes && !c->pass_head; --k)  // (the head pass zeroes them)
-    TT_CUDA(c, cudaMemsetAsync(k == l ? Yl : Ys, 0, sizeof(float) * (size_t)c->J * c->n[k], c->stream));
+    if ((k == l ? a.cl : a.cs) == 1)
+      TT_CUDA(c, cudaMemsetAsync(k == l ? Yl : Ys, 0, sizeof(float) * (size_t)c->J * c->n[k], c->stream));
+  const bool copies = a.cs > 1 || a.cl > 1;
+  if (copies && !c->ysl_zero)
+    TT_CUDA(c, cudaMemsetAsync(c->d_ysl, 0, sizeof(float) * (size_t)tt_tail_copies(c), c->stream));
+  if (copies) c->ysl_zero = false;
   a.E = c->stride[c->d - c->tail_modes];
   a.J = c->J;
   a.n0 = (int)c->n[0];
@@ -929,11 +1019,19 @@ int tt_launch_tail_pass(tt_ctx* c, const void* A, const float* scales, float* Ys
   a.ns = c->tail_modes == 2 ? (int)c->n[s] : 1;
   a.nl = (int)c->n[l];
   switch (c->dtype) {
-    case TT_F64: return launch_tail<TT_F64>(c, a);
-    case TT_F32: return launch_tail<TT_F32>(c, a);
-    case TT_BF16: return launch_tail<TT_BF16>(c, a);
-    default: return launch_tail<TT_FP8E4M3>(c, a);
+    case TT_F64: TT_TRY(launch_tail<TT_F64>(c, a)); break;
+    case TT_F32: TT_TRY(launch_tail<TT_F32>(c, a)); break;
+    case TT_BF16: TT_TRY(launch_tail<TT_BF16>(c, a)); break;
+    default: TT_TRY(launch_tail<TT_FP8E4M3>(c, a)); break;
   }
+  if (!copies) return TT_OK;
+  TailOutArgs o{};
+  if (a.cs > 1) o.src[0] = a.Ys, o.dst[0] = Ys, o.n[0] = ls, o.copies[0] = a.cs;
+  if (a.cl > 1) o.src[1] = a.Yl, o.dst[1] = Yl, o.n[1] = ll, o.copies[1] = a.cl;
+  k_tail_out<<<(int)std::min<int64_t>((std::max(o.n[0], o.n[1]) + 255) / 256, 8 * tt_sm_count()), 256, 0, c->stream>>>(o);
+  TT_LAUNCH(c, "k_tail_out");
+  c->ysl_zero = true;
+  return TT_OK;
 }
 
 // The data sketches of all modes on c->stream: the passes, then one launch per remaining mode; ev[k]

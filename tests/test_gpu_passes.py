@@ -142,3 +142,31 @@ def test_a_workspace_cap_that_leaves_no_room_for_the_passes():
     for a, b in zip(*Y):
         assert float(torch.linalg.vector_norm(a - b)) <= TOL * float(torch.linalg.vector_norm(a))
     ctx.close()
+
+
+# Rounding of FP32 sums: n adds one after the other, each off by at most 2^-24 of the partial sum, leave a
+# relative error of at most about 2^-24 sqrt(n / 2) of a sum of n terms of random sign (the partial sums
+# grow with the square root); the levels of a sum (a bucket's entries of one slab, the slabs of one copy,
+# the copies in pairs) add in squares.
+def _chain_bound(*levels):
+    return 2.0**-24 * np.sqrt(sum(n / 2 for n in levels))
+
+
+@pytest.mark.parametrize("dims,levels", [
+    ((64, 170, 2, 400), (11, 25, 10)),  # Y_2: 800 slabs and chunks per bucket, 32 copies
+    ((64, 170, 400, 2), (11, 25, 10)),  # Y_3: its registers' runs cut, 8 copies
+])
+def test_long_tail_sums_keep_their_accuracy(dims, levels):
+    """Few columns and many slabs of two chunks: a bucket of the last two modes sums 800 slab chunks."""
+    J, seed = 512, 977
+    a = synth.random_tensor(dims, 31)
+    flat, _, exact = synth.quantize(a, "f32")
+    ctx = lib.Context(dims, [1, 2, 2, 2, 1], J, 1e-3, seed)
+    Y = [torch.empty(n, J, device="cuda") for n in dims]
+    ctx.tt_sketch_unfold(lib.device_tensor(flat, "f32"), -1, 5, Y)
+    hs, vs = O.draw_sketch(seed, 5, dims, J)
+    k = 2 if dims[2] == 2 else 3
+    ref = np.stack([O.sketch_unfolding_column(exact, hs, vs, J, k, i) for i in range(2)])
+    err = np.linalg.norm(Y[k].double().cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert err <= _chain_bound(*levels), err
+    ctx.close()

@@ -690,7 +690,7 @@ static void tt_workspace_each(tt_ctx* c, F&& A) {
     }
     A((void**)&c->d_rkey, sizeof(int32_t) * c->R[1]);
     A((void**)&c->spare.rkey, sizeof(int32_t) * c->R[1]);
-    A((void**)&c->d_y01, sizeof(float) * c->J * (size_t)(c->p0 + c->p1));
+    A((void**)&c->d_y01, sizeof(float) * (size_t)tt_head_copies(c));
   }
   if (c->pass_tail) {
     const size_t e = sizeof(uint16_t) * 4 * (size_t)c->tail_blocks * c->tail_nchunk;
@@ -881,7 +881,7 @@ extern "C" int tt_sketch_init(tt_ctx** out, const tt_params* p, void* stream) {
     e = cudaMemcpyAsync(c->d_twstage, tws.data(), sizeof(float2) * tws.size(), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
   if (e == cudaSuccess && c->d_y01)
-    e = cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)c->J * (c->p0 + c->p1), c->stream);
+    e = cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)tt_head_copies(c), c->stream);
   if (e == cudaSuccess && c->d_ysl) e = cudaMemsetAsync(c->d_ysl, 0, sizeof(float) * (size_t)tt_tail_copies(c), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {

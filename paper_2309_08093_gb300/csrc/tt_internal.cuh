@@ -144,7 +144,8 @@ struct tt_ctx {
   uint16_t* d_tlist = nullptr;          // tail pass: the head's entries by bucket, chunk after chunk
   uint32_t* d_tbucket = nullptr;        // tail pass: bucket words (J per chunk), then sign words
   bool pass_valid = false;              // d_hplan, d_tlist, d_tbucket are those of the current draw
-  float* d_y01 = nullptr;               // J x p0 then J x p1: Y_0 and Y_1 by rows (zero between head passes)
+  int head_c0 = 1, head_c1 = 1;         // copies of Y_0 and Y_1 that the head pass adds into (powers of two)
+  float* d_y01 = nullptr;               // those copies by rows, J x p0 then J x p1 (zero between head passes)
   bool y01_zero = true;                 // they are (false after a launch that failed in between)
   float* d_ysl = nullptr;               // tail_cs copies of Y_s, then tail_cl of Y_l, those above one (zero likewise)
   bool ysl_zero = true;
@@ -318,6 +319,7 @@ int tt_launch_unfold_planned(tt_ctx* c, const void* A, const float* scales, int 
 // allows, tt_launch_unfold for the other modes; ev[k] (optional) is recorded after Y[k]
 int tt_launch_unfold_all(tt_ctx* c, const void* A, const float* scales, float* const* Y, cudaEvent_t* ev = nullptr);
 void tt_pass_plan(tt_ctx* c);                 // which modes the passes cover, from the shape
+int64_t tt_head_copies(const tt_ctx* c);      // floats of d_y01
 int64_t tt_tail_copies(const tt_ctx* c);      // floats of d_ysl
 unsigned tt_pass_mask(const tt_ctx* c, const void* A);   // modes of A covered by the passes
 unsigned tt_pass_plans(const tt_ctx* c, const void* A);  // modes whose fibre plan tt_launch_unfold_all reads

@@ -42,8 +42,9 @@ __device__ __forceinline__ float take_copies(float* p, int64_t stride, int n) {
   return isfinite(e) ? s + e : s;  // (an infinite sum has no error term)
 }
 
-// copies of an accumulator whose entries take `adds` FP32 adds one after the other: about sqrt(adds), a
-// power of two, so that the adds to a copy and the copies are two short sums
+// Copies of an accumulator whose entries take `adds` FP32 adds one after the other: about sqrt(adds), a
+// power of two, which leaves an entry no more rounding than the sums of one launch per mode (register runs,
+// a column copy per work item, Y_k). FP8, whose runs are exact there, asks for more by larger `adds`.
 int copies_of(double adds) {
   int c = 1;
   while (2.0 * c * c < adds && c < 64) c *= 2;  // nearest power of two on a logarithmic scale
@@ -60,8 +61,9 @@ struct HeadArgs {
   const int32_t* key;    // c of each plan entry
   const int32_t *h0, *h1;
   const int8_t *v0, *v1;
-  float* Y0r;  // J x p0, row b = bucket b of Y_0
-  float* Y1r;  // J x p1, row b = bucket b of Y_1
+  float* Y0r;  // c0 copies of J x p0, row b = bucket b of Y_0 (FP8: before the finite scales)
+  float* Y1r;  // c1 copies of J x p1, row b = bucket b of Y_1
+  int c0, c1;  // powers of two
   int64_t R;   // slabs
   int J, n0, n1, p0, p1;
   int G1, nch;  // columns i_1 per chunk of a slab, chunks
@@ -138,14 +140,20 @@ __device__ __forceinline__ void head_add(const uint32_t* w, float s, float* acc)
   }
 }
 
-// Bound: DRAM while runs are long (100^4 FP32, J = 1024, 9.8 slabs per run: 80 us, 5.0 TB/s), the
-// flushes' L2 atomics and tile traffic beside it when they are short (J = 4096, 2.4 slabs per run:
-// 113 us for both modes, 206 us with one launch per mode). The flushes go to L2 as 16-byte atomic adds
+// Bound: DRAM while runs are long (100^4 FP32, J = 1024, 9.8 slabs per run: 98 us with k_head_out, 170 us
+// with one launch per mode), the flushes' L2 atomics and tile traffic beside it when they are short
+// (J = 4096, 2.4 slabs per run: 132 and 206 us). The flushes go to L2 as 16-byte atomic adds
 // along rows (5.9 TB/s of sums, measured alone) because shared-memory float atomics at random
 // buckets sustain half of that (0.75 T adds/s) and need a copy of the columns per CTA. Two CTAs per
 // SM: one flushes while the other loads.
 // A slab's chunk is read as a run of VB-byte vectors, whatever columns they lie in: thread t holds
 // the vectors t + T j. U slabs are loaded ahead of the sums.
+// Accuracy: a bucket of Y_0 (Y_1) takes about runs * n_1 / J (runs * n_0 / J) of these adds one after the
+// other, and the rounding error of FP32 sums grows with their square root; so segments add to one of c0
+// (c1) copies of the rows in turn, and k_head_out adds the copies up. FP8 rows of Y_0 are summed before
+// their scales, exactly while |sums| < 2^15. (One sum per row: 83 and 126 us.) Relative error, one sum / copies / one launch per mode:
+// Y_1 of 100^4 FP32 1.8e-7 / 8.2e-8 / 9.5e-8, Y_0 of 256 x 256 x 3 x 128 FP32 1.3e-7 / 5.8e-8 / 8.9e-8,
+// of 40^5 FP8 1.3e-7 / 2.5e-8 / 4.6e-8.
 template <int DT, int VB>
 __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
   constexpr int EB = TtElem<DT>::bytes;
@@ -163,14 +171,14 @@ __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
   const int rows_tile = (a.G1 + 3) & ~3, n0p = (n0 + 3) & ~3;
   float* tile = hsm;                                        // rows_tile x pitch
   float* cf0 = tile + (size_t)rows_tile * pitch;            // n0p: v_0 (times the FP8 scale)
-  float* sc0 = cf0 + n0p;                                   // n0p: FP8 scale (1 otherwise)
+  float* sc0 = cf0 + n0p;                                   // n0p: what of the FP8 scale k_head_out leaves
   int* hh0 = reinterpret_cast<int*>(sc0 + n0p);             // n0p
   int* hh1 = hh0 + n0p;                                     // rows_tile: h_1, sign in bit 31
   uint32_t* sw = reinterpret_cast<uint32_t*>(hh1 + rows_tile);  // HEAD_BATCH
   int* sk = reinterpret_cast<int*>(sw + HEAD_BATCH);        // HEAD_BATCH
   for (int i = t; i < n0p; i += T) {
     const float s = a.scales && i < n0 ? __ldg(a.scales + i) : 1.f;
-    sc0[i] = s;
+    sc0[i] = isfinite(s) ? 1.f : s;
     cf0[i] = i < n0 && __ldg(a.v0 + i) < 0 ? -s : s;
     hh0[i] = i < n0 ? __ldg(a.h0 + i) : 0;
   }
@@ -180,6 +188,8 @@ __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
   const int ne = n0 * g1;  // entries of a slab's chunk
   const char* base = a.A + (int64_t)c0 * n0 * EB + (int64_t)t * VB;
   const int64_t fb = (int64_t)n0 * EB;
+  float* const y0r = a.Y0r + (int64_t)(seg & (a.c0 - 1)) * J * a.p0;
+  float* const y1r = a.Y1r + (int64_t)(seg & (a.c1 - 1)) * J * a.p1;
   const bool quads = EPV >= 4 && (n0 & 3) == 0;  // every four entries lie in one column
   float acc[NV][EPV];
 #pragma unroll
@@ -205,7 +215,7 @@ __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
               *reinterpret_cast<float4*>(tile + tile_at(i1, i0, pitch)) = z;
               float4 m = make_float4(s1 * z.x, s1 * z.y, s1 * z.z, s1 * z.w);
               if (DT == TT_FP8E4M3) m.x *= sc0[i0], m.y *= sc0[i0 + 1], m.z *= sc0[i0 + 2], m.w *= sc0[i0 + 3];
-              red4(a.Y0r + (int64_t)tt_modj(c + (hw & 0x7FFFFFFF), J) * a.p0 + i0, m);
+              red4(y0r + (int64_t)tt_modj(c + (hw & 0x7FFFFFFF), J) * a.p0 + i0, m);
             }
           }
     } else {
@@ -233,7 +243,7 @@ __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
       if (i0 < n0 && i1 < g1p) {
         const float* src = tile + tile_at(i1, i0, pitch);  // columns i1 .. i1 + 3 share the swizzle
         const float s = cf0[i0];
-        red4(a.Y1r + (int64_t)tt_modj(c + hh0[i0], J) * a.p1 + c0 + i1,
+        red4(y1r + (int64_t)tt_modj(c + hh0[i0], J) * a.p1 + c0 + i1,
              make_float4(s * src[0], s * src[pitch], s * src[2 * pitch], s * src[3 * pitch]));
       }
     }
@@ -245,7 +255,7 @@ __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
         const float4 z = *reinterpret_cast<const float4*>(tile + tile_at(i1, i0, pitch));
         float4 m = make_float4(s1 * z.x, s1 * z.y, s1 * z.z, s1 * z.w);
         if (DT == TT_FP8E4M3) m.x *= sc0[i0], m.y *= sc0[i0 + 1], m.z *= sc0[i0 + 2], m.w *= sc0[i0 + 3];
-        red4(a.Y0r + (int64_t)tt_modj(c + (hw & 0x7FFFFFFF), J) * a.p0 + i0, m);
+        red4(y0r + (int64_t)tt_modj(c + (hw & 0x7FFFFFFF), J) * a.p0 + i0, m);
       }
   };
 
@@ -286,28 +296,26 @@ __global__ void __launch_bounds__(HEAD_TMAX, 2) k_head_pass(HeadArgs a) {
   if (cur >= 0) flush(cur);
 }
 
-// Y_0 and Y_1 (column-major, J x n) from the row-major J x p accumulators, 32 x 32 tiles; the
-// accumulators are left zero for the next head pass
-__global__ void __launch_bounds__(256) k_head_out(float* __restrict__ Y0r, float* __restrict__ Y1r, float* __restrict__ Y0, float* __restrict__ Y1, int J, int n0,
-                                                   int n1, int p0, int p1, int tiles0) {
+// Y_0 and Y_1 (column-major, J x n) from the copies of the row-major J x p accumulators, 32 x 32 tiles;
+// the accumulators are left zero for the next head pass
+struct HeadOutArgs {
+  float *Y0r, *Y1r, *Y0, *Y1;
+  const float* scales;  // of Y_0's columns (null: none)
+  int J, n0, n1, p0, p1, c0, c1, tiles0;
+};
+__global__ void __launch_bounds__(1024) k_head_out(HeadOutArgs a) {
   __shared__ float tl[32][33];
-  const bool first = (int)blockIdx.y < tiles0;
-  float* src = first ? Y0r : Y1r;
-  float* dst = first ? Y0 : Y1;
-  const int n = first ? n0 : n1, p = first ? p0 : p1;
-  const int i0 = 32 * ((int)blockIdx.y - (first ? 0 : tiles0)), b0 = 32 * blockIdx.x;
+  const bool first = (int)blockIdx.y < a.tiles0;
+  const int n = first ? a.n0 : a.n1, p = first ? a.p0 : a.p1, J = a.J;
+  const int i0 = 32 * ((int)blockIdx.y - (first ? 0 : a.tiles0)), b0 = 32 * blockIdx.x;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-#pragma unroll
-  for (int r = y; r < 32; r += 8)
-    if (b0 + r < J && i0 + x < n) {
-      float* q = src + (int64_t)(b0 + r) * p + i0 + x;
-      tl[r][x] = *q;
-      *q = 0.f;
-    }
+  if (b0 + y < J && i0 + x < n) {
+    float s = first && a.scales ? __ldg(a.scales + i0 + x) : 1.f;
+    if (!isfinite(s)) s = 1.f;  // (k_head_pass applied it)
+    tl[y][x] = s * take_copies((first ? a.Y0r : a.Y1r) + (int64_t)(b0 + y) * p + i0 + x, (int64_t)J * p, first ? a.c0 : a.c1);
+  }
   __syncthreads();
-#pragma unroll
-  for (int r = y; r < 32; r += 8)
-    if (b0 + x < J && i0 + r < n) dst[(int64_t)(i0 + r) * J + b0 + x] = tl[x][r];
+  if (b0 + x < J && i0 + y < n) (first ? a.Y0 : a.Y1)[(int64_t)(i0 + y) * J + b0 + x] = tl[x][y];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -795,18 +803,41 @@ int launch_tail(tt_ctx* c, const TailArgs& a) {
   }
 }
 
+int head_cols(const tt_ctx* c) {  // columns i_1 per chunk
+  // at most what the threads hold, and 128 KB of transposition tile
+  const int64_t cap = std::min<int64_t>(HEAD_TMAX * (c->dtype == TT_F64 ? head_acc<TT_F64>() : head_acc<TT_F32>()) / c->n[0],
+                                        (128 * 1024 / 4) / ((c->n[0] + 31) & ~31));
+  if (cap >= c->n[1]) return (int)c->n[1];
+  const int64_t nch = (c->n[1] + (cap & ~3) - 1) / std::max<int64_t>(4, cap & ~3);
+  return (int)(((c->n[1] + nch - 1) / nch + 3) & ~3);
+}
+
+struct HeadGeom {
+  int G1, nch, threads;
+  size_t smem;
+  int per_sm;  // CTAs per SM, at most
+};
+HeadGeom head_geom(const tt_ctx* c) {
+  HeadGeom g;
+  g.G1 = head_cols(c);
+  g.nch = (int)((c->n[1] + g.G1 - 1) / g.G1);
+  const int per_warp = 32 * (c->dtype == TT_F64 ? head_acc<TT_F64>() : head_acc<TT_F32>());  // entries
+  g.threads = (int)((c->n[0] * g.G1 + per_warp - 1) / per_warp) * 32;
+  const size_t rows = (size_t)((g.G1 + 3) & ~3), pitch = (size_t)((c->n[0] + 31) & ~31);
+  g.smem = sizeof(float) * (rows * pitch + 3 * (size_t)c->p0 + rows + 2 * HEAD_BATCH);
+  g.per_sm = std::max(1, std::min({32, 2 * HEAD_TMAX / g.threads, (int)(228 * 1024 / (g.smem + 1024))}));
+  return g;
+}
+
 template <int DT, int VB>
 int launch_head_vb(tt_ctx* c, HeadArgs a) {
-  constexpr int PT = 32 * head_acc<DT>();  // entries per warp
-  const int threads = (int)(((int64_t)a.n0 * a.G1 + PT - 1) / PT) * 32;
-  const int rows = (a.G1 + 3) & ~3;
-  const size_t smem = sizeof(float) * ((size_t)rows * a.pitch + 3 * (size_t)((a.n0 + 3) & ~3) + rows + 2 * HEAD_BATCH);
+  const HeadGeom g = head_geom(c);
   auto kern = k_head_pass<DT, VB>;
-  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
   int per_sm = 1;
-  TT_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
-  a.nseg = (int)std::max<int64_t>(1, std::min<int64_t>(a.R, pass_ctas(c, per_sm) / a.nch));
-  kern<<<a.nseg * a.nch, threads, smem, c->stream>>>(a);
+  TT_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, g.threads, g.smem));
+  a.nseg = (int)std::max<int64_t>(1, std::min<int64_t>(a.R, pass_ctas(c, std::min(per_sm, g.per_sm)) / a.nch));
+  kern<<<a.nseg * a.nch, g.threads, g.smem, c->stream>>>(a);
   TT_LAUNCH(c, "k_head_pass");
   return TT_OK;
 }
@@ -822,15 +853,6 @@ int launch_head(tt_ctx* c, const HeadArgs& a) {
     if (at % 4 == 0) return launch_head_vb<DT, 4>(c, a);
   if constexpr (EB < 4) return launch_head_vb<DT, EB>(c, a);
   return tt_fail(c, TT_EINVAL, "A is not aligned to its storage type");
-}
-
-int head_cols(const tt_ctx* c) {  // columns i_1 per chunk
-  // at most what the threads hold, and 128 KB of transposition tile
-  const int64_t cap = std::min<int64_t>(HEAD_TMAX * (c->dtype == TT_F64 ? head_acc<TT_F64>() : head_acc<TT_F32>()) / c->n[0],
-                                        (128 * 1024 / 4) / ((c->n[0] + 31) & ~31));
-  if (cap >= c->n[1]) return (int)c->n[1];
-  const int64_t nch = (c->n[1] + (cap & ~3) - 1) / std::max<int64_t>(4, cap & ~3);
-  return (int)(((c->n[1] + nch - 1) / nch + 3) & ~3);
 }
 
 // entries per chunk: what a CTA's threads can fetch at once (JJ loads each). FP8 slabs on 4-byte
@@ -851,21 +873,34 @@ bool tail_takes(const tt_ctx* c, const void* A) {
 // Which modes the passes cover, from the shape alone. Workspaces of both sketch draws follow from it.
 // The head pass needs slabs that fill a CTA's warps (512 entries) and columns that leave room for four
 // in a chunk; its row accumulators stay in L2 (32 MB). The tail pass needs chunks of at least that
-// size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. J up to 8192:
-// eight buckets per thread. The deterministic mode has its own kernels; the batch autotuner times
-// launches per mode.
+// size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. Where the copies
+// of a pass would pass 96 MB each mode takes half as many, and where those would, no pass: with fewer its
+// sums would be off by more than those of one launch per mode. J up to 8192: eight buckets per thread.
+// The deterministic mode has its own kernels; the batch autotuner times launches per mode.
 void tt_pass_plan(tt_ctx* c) {
   c->pass_head = c->pass_tail = false;
   c->tail_modes = 0;
   if (c->det || (c->flags & TT_FLAG_BATCH_AUTOTUNE) || c->J > 8192) return;
   const int64_t e2 = c->n[0] * c->n[1];
+  const bool fp8 = c->dtype == TT_FP8E4M3;
   c->p0 = (int)((c->n[0] + 3) & ~3);
   c->p1 = (int)((c->n[1] + 3) & ~3);
   c->pass_head = e2 >= 512 && c->n[0] <= HEAD_TMAX * head_acc<TT_F64>() / 4 && (int64_t)c->J * (c->p0 + c->p1) <= (8 << 20);
+  if (c->pass_head) {
+    const HeadGeom g = head_geom(c);
+    const double R = (double)c->N / e2, segs = std::max(1.0, std::min(R, 152.0 * g.per_sm / g.nch));  // (152 SMs)
+    const double runs = c->J * -std::expm1(-R / c->J) + segs;  // groups c that slabs have, and cut ones
+    const double cap = segs * segs, adds0 = runs * c->n[1] / c->J, adds1 = (fp8 ? 2 : 1) * runs * c->n[0] / c->J;
+    c->pass_head = false;
+    for (double part = 1.0; part >= 0.5 && !c->pass_head; part /= 2) {
+      c->head_c0 = fp8 ? 1 : copies_of(part * std::min(cap, adds0));
+      c->head_c1 = copies_of(part * std::min(cap, adds1));
+      c->pass_head = tt_head_copies(c) <= PASS_COPIES_MAX;
+    }
+  }
   const int nt = c->d >= 4 ? 2 : c->d == 3 ? 1 : 0;
   if (nt) {
     const int64_t E = c->stride[c->d - nt];
-    const bool fp8 = c->dtype == TT_FP8E4M3;
     // the longest chunk, halved until an SM's shared memory holds it (long FP8 rows bring a scale each)
     bool fits = false;
     for (int64_t cm = tail_chunk_max(c, E); !fits && cm >= 2048; cm /= 2) {
@@ -877,16 +912,24 @@ void tt_pass_plan(tt_ctx* c) {
     }
     c->pass_tail = fits && E >= 512 && E * 8 >= c->J && c->tail_nchunk <= 64;
     if (c->pass_tail) {
-      const double slabs = (double)c->tail_nchunk * c->n[c->d - 1];  // that a bucket of Y_s meets
-      c->tail_cs = nt == 2 ? copies_of((fp8 ? 2.0 : 1.0) * slabs * -std::expm1(-(double)c->tail_chunk / c->J)) : 1;
       const int run = tail_run(c->dtype);
-      c->tail_cl = copies_of((fp8 ? 3.0 : 2.0) * c->tail_nchunk * (nt == 2 ? (c->n[c->d - 2] + run - 1) / run : 1));
+      const double slabs = (double)c->tail_nchunk * c->n[c->d - 1];  // that a bucket of Y_s meets
+      const double adds_s = (fp8 ? 2 : 1) * slabs * -std::expm1(-(double)c->tail_chunk / c->J);
+      const double adds_l = (fp8 ? 3 : 2) * (double)c->tail_nchunk * (nt == 2 ? (c->n[c->d - 2] + run - 1) / run : 1);
+      c->pass_tail = false;
       c->tail_modes = nt;
-      if (tt_tail_copies(c) > PASS_COPIES_MAX) c->pass_tail = false, c->tail_modes = 0;
+      for (double part = 1.0; part >= 0.5 && !c->pass_tail; part /= 2) {
+        c->tail_cs = nt == 2 ? copies_of(part * adds_s) : 1;
+        c->tail_cl = copies_of(part * adds_l);
+        c->pass_tail = tt_tail_copies(c) <= PASS_COPIES_MAX;
+      }
+      if (!c->pass_tail) c->tail_modes = 0;
     }
   }
   c->head_sorted = c->pass_head && c->N / e2 <= HEAD_PLAN_MAX;
 }
+
+int64_t tt_head_copies(const tt_ctx* c) { return (int64_t)c->J * (c->head_c0 * c->p0 + c->head_c1 * c->p1); }
 
 int64_t tt_tail_copies(const tt_ctx* c) {
   int64_t n = 0;
@@ -958,9 +1001,12 @@ int tt_launch_head_pass(tt_ctx* c, const void* A, const float* scales, float* co
   a.p0 = c->p0;
   a.p1 = c->p1;
   a.Y0r = c->d_y01;
-  a.Y1r = c->d_y01 + (int64_t)c->J * c->p0;
-  a.G1 = head_cols(c);
-  a.nch = (a.n1 + a.G1 - 1) / a.G1;
+  a.Y1r = c->d_y01 + (int64_t)c->head_c0 * c->J * c->p0;
+  a.c0 = c->head_c0;
+  a.c1 = c->head_c1;
+  const HeadGeom g = head_geom(c);
+  a.G1 = g.G1;
+  a.nch = g.nch;
   a.pitch = (a.n0 + 31) & ~31;
   a.inv_n0 = (uint32_t)((((uint64_t)1 << 32) + a.n0 - 1) / a.n0);
   for (int z = 0; z < c->tail_modes; ++z)
@@ -968,7 +1014,7 @@ int tt_launch_head_pass(tt_ctx* c, const void* A, const float* scales, float* co
       a.zero[z] = Y[c->d - 1 - z];
       a.nzero[z] = (int64_t)c->J * c->n[c->d - 1 - z];
     }
-  if (!c->y01_zero) TT_CUDA(c, cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)c->J * (c->p0 + c->p1), c->stream));
+  if (!c->y01_zero) TT_CUDA(c, cudaMemsetAsync(c->d_y01, 0, sizeof(float) * (size_t)tt_head_copies(c), c->stream));
   c->y01_zero = false;
   switch (c->dtype) {
     case TT_F64: TT_TRY(launch_head<TT_F64>(c, a)); break;
@@ -976,8 +1022,9 @@ int tt_launch_head_pass(tt_ctx* c, const void* A, const float* scales, float* co
     case TT_BF16: TT_TRY(launch_head<TT_BF16>(c, a)); break;
     default: TT_TRY(launch_head<TT_FP8E4M3>(c, a)); break;
   }
-  const int t0 = (a.n0 + 31) / 32, t1 = (a.n1 + 31) / 32;
-  k_head_out<<<dim3((c->J + 31) / 32, t0 + t1), 256, 0, c->stream>>>(a.Y0r, a.Y1r, Y[0], Y[1], c->J, a.n0, a.n1, a.p0, a.p1, t0);
+  const HeadOutArgs o = {a.Y0r, a.Y1r, Y[0], Y[1], c->dtype == TT_FP8E4M3 ? scales : nullptr,
+                         c->J,  a.n0,  a.n1, a.p0, a.p1, a.c0, a.c1, (a.n0 + 31) / 32};
+  k_head_out<<<dim3((c->J + 31) / 32, o.tiles0 + (a.n1 + 31) / 32), 1024, 0, c->stream>>>(o);
   TT_LAUNCH(c, "k_head_out");
   c->y01_zero = true;
   return TT_OK;

@@ -152,21 +152,23 @@ def _chain_bound(*levels):
     return 2.0**-24 * np.sqrt(sum(n / 2 for n in levels))
 
 
-@pytest.mark.parametrize("dims,levels", [
-    ((64, 170, 2, 400), (11, 25, 10)),  # Y_2: 800 slabs and chunks per bucket, 32 copies
-    ((64, 170, 400, 2), (11, 25, 10)),  # Y_3: its registers' runs cut, 8 copies
+@pytest.mark.parametrize("dims,J,dtype,k,levels", [
+    ((64, 170, 2, 400), 512, "f32", 2, (11, 25, 10)),  # 800 slab chunks per bucket, 32 copies
+    ((64, 170, 400, 2), 512, "f32", 3, (11, 25, 10)),  # its registers' runs cut, 8 copies
+    ((40, 16, 90, 60), 64, "f32", 0, (2, 25, 1)),      # 3,100 runs of 16 columns: 775 adds, 32 copies
+    ((40, 16, 90, 60), 64, "f32", 1, (2, 61, 1)),      # ... of 40 rows: 1,940 adds, 32 copies
+    ((40, 16, 90, 60), 64, "fp8", 0, (2, 2, 1)),       # sums of unscaled FP8 entries are exact
 ])
-def test_long_tail_sums_keep_their_accuracy(dims, levels):
-    """Few columns and many slabs of two chunks: a bucket of the last two modes sums 800 slab chunks."""
-    J, seed = 512, 977
-    a = synth.random_tensor(dims, 31)
-    flat, _, exact = synth.quantize(a, "f32")
-    ctx = lib.Context(dims, [1, 2, 2, 2, 1], J, 1e-3, seed)
+def test_long_sums_keep_their_accuracy(dims, J, dtype, k, levels):
+    """Few columns and many slabs: buckets that take hundreds of adds."""
+    seed = 977
+    flat, scales, exact = synth.quantize(synth.random_tensor(dims, 31), dtype)
+    ctx = lib.Context(dims, [1, 2, 2, 2, 1], J, 1e-3, seed, dtype)
     Y = [torch.empty(n, J, device="cuda") for n in dims]
-    ctx.tt_sketch_unfold(lib.device_tensor(flat, "f32"), -1, 5, Y)
+    sc = torch.from_numpy(scales).cuda() if scales is not None else None
+    ctx.tt_sketch_unfold(lib.device_tensor(flat, dtype), -1, 5, Y, sc)
     hs, vs = O.draw_sketch(seed, 5, dims, J)
-    k = 2 if dims[2] == 2 else 3
     ref = np.stack([O.sketch_unfolding_column(exact, hs, vs, J, k, i) for i in range(2)])
-    err = np.linalg.norm(Y[k].double().cpu().numpy() - ref) / np.linalg.norm(ref)
+    err = np.linalg.norm(Y[k][:2].double().cpu().numpy() - ref) / np.linalg.norm(ref)
     assert err <= _chain_bound(*levels), err
     ctx.close()

@@ -42,12 +42,12 @@ __device__ __forceinline__ float take_copies(float* p, int64_t stride, int n) {
   return isfinite(e) ? s + e : s;  // (an infinite sum has no error term)
 }
 
-// Copies of an accumulator whose entries take `adds` FP32 adds one after the other: about sqrt(adds), a
+// Copies of an accumulator whose entries take `adds` FP32 adds one after the other: about 0.8 sqrt(adds), a
 // power of two, which leaves an entry no more rounding than the sums of one launch per mode (register runs,
 // a column copy per work item, Y_k). FP8, whose runs are exact there, asks for more by larger `adds`.
 int copies_of(double adds) {
   int c = 1;
-  while (2.0 * c * c < adds && c < 64) c *= 2;  // nearest power of two on a logarithmic scale
+  while (3.0 * c * c < adds && c < 64) c *= 2;
   return c;
 }
 
@@ -352,7 +352,9 @@ struct PassPlanArgs {
   int32_t* key;
 };
 constexpr int64_t HEAD_PLAN_MAX = 1 << 15;
-constexpr int64_t PASS_COPIES_MAX = 24 << 20;  // floats of a pass's accumulators (they are to stay in L2)
+// floats of a pass's accumulators, 48 MB: they are to stay in L2 beside A (300 x 300 x 33 x 33 at J = 8192
+// with 79 MB: head pass 359 us, one launch per mode 312)
+constexpr int64_t PASS_COPIES_MAX = 12 << 20;
 
 __global__ void __launch_bounds__(1024) k_pass_plans(PassPlanArgs a) {
   extern __shared__ int psm[];  // J counts, then cursors
@@ -874,7 +876,7 @@ bool tail_takes(const tt_ctx* c, const void* A) {
 // The head pass needs slabs that fill a CTA's warps (512 entries) and columns that leave room for four
 // in a chunk; its row accumulators stay in L2 (32 MB). The tail pass needs chunks of at least that
 // size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. Where the copies
-// of a pass would pass 96 MB each mode takes half as many, and where those would, no pass: with fewer its
+// of a pass exceed 48 MB each mode takes half as many, and where those do, no pass: with fewer its
 // sums would be off by more than those of one launch per mode. J up to 8192: eight buckets per thread.
 // The deterministic mode has its own kernels; the batch autotuner times launches per mode.
 void tt_pass_plan(tt_ctx* c) {
@@ -890,7 +892,7 @@ void tt_pass_plan(tt_ctx* c) {
     const HeadGeom g = head_geom(c);
     const double R = (double)c->N / e2, segs = std::max(1.0, std::min(R, 152.0 * g.per_sm / g.nch));  // (152 SMs)
     const double runs = c->J * -std::expm1(-R / c->J) + segs;  // groups c that slabs have, and cut ones
-    const double cap = segs * segs, adds0 = runs * c->n[1] / c->J, adds1 = (fp8 ? 2 : 1) * runs * c->n[0] / c->J;
+    const double cap = segs * segs, adds0 = runs * c->n[1] / c->J, adds1 = (fp8 ? 1.9 : 1.0) * runs * c->n[0] / c->J;
     c->pass_head = false;
     for (double part = 1.0; part >= 0.5 && !c->pass_head; part /= 2) {
       c->head_c0 = fp8 ? 1 : copies_of(part * std::min(cap, adds0));
@@ -914,8 +916,8 @@ void tt_pass_plan(tt_ctx* c) {
     if (c->pass_tail) {
       const int run = tail_run(c->dtype);
       const double slabs = (double)c->tail_nchunk * c->n[c->d - 1];  // that a bucket of Y_s meets
-      const double adds_s = (fp8 ? 2 : 1) * slabs * -std::expm1(-(double)c->tail_chunk / c->J);
-      const double adds_l = (fp8 ? 3 : 2) * (double)c->tail_nchunk * (nt == 2 ? (c->n[c->d - 2] + run - 1) / run : 1);
+      const double adds_s = (fp8 ? 3 : 1) * slabs * -std::expm1(-(double)c->tail_chunk / c->J);
+      const double adds_l = (fp8 ? 4 : 1) * (double)c->tail_nchunk * (nt == 2 ? (c->n[c->d - 2] + run - 1) / run : 1);
       c->pass_tail = false;
       c->tail_modes = nt;
       for (double part = 1.0; part >= 0.5 && !c->pass_tail; part /= 2) {

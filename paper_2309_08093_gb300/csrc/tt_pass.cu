@@ -878,11 +878,13 @@ bool tail_takes(const tt_ctx* c, const void* A) {
 // size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. Where the copies
 // of a pass exceed 48 MB each mode takes half as many, and where those do, no pass: with fewer its
 // sums would be off by more than those of one launch per mode. J up to 8192: eight buckets per thread.
+// One row per slab column (n_0 = 1) goes one launch per mode: the passes divide entry numbers by n_0 with a
+// multiplication by 2^32 / n_0, which has no 32-bit value then.
 // The deterministic mode has its own kernels; the batch autotuner times launches per mode.
 void tt_pass_plan(tt_ctx* c) {
   c->pass_head = c->pass_tail = false;
   c->tail_modes = 0;
-  if (c->det || (c->flags & TT_FLAG_BATCH_AUTOTUNE) || c->J > 8192) return;
+  if (c->det || (c->flags & TT_FLAG_BATCH_AUTOTUNE) || c->J > 8192 || c->n[0] == 1) return;
   const int64_t e2 = c->n[0] * c->n[1];
   const bool fp8 = c->dtype == TT_FP8E4M3;
   c->p0 = (int)((c->n[0] + 3) & ~3);

@@ -69,6 +69,16 @@ def test_all_modes_against_the_oracle(dims, J, dtype):
     _check(dims, J, dtype)
 
 
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16", "fp8"])
+@pytest.mark.parametrize("dims,J", [
+    ((1, 600, 5), 64), ((1, 32, 32, 8, 8), 256), ((1, 700, 3, 4), 512),  # first mode
+    ((600, 1, 5), 64), ((32, 24, 1, 9), 256), ((24, 23, 1, 7, 5), 512),  # a middle one
+    ((40, 30, 1), 64), ((32, 24, 9, 1), 256), ((1, 1, 600), 32), ((600, 1, 1, 1), 32),  # the last, several
+])
+def test_modes_of_size_one(dims, J, dtype):
+    _check(dims, J, dtype, rank=1)
+
+
 @pytest.mark.parametrize("dtype,offset", [("f32", 1), ("f32", 2), ("f64", 1), ("bf16", 1), ("bf16", 2), ("bf16", 4),
                                           ("fp8", 1), ("fp8", 2), ("fp8", 4), ("fp8", 8)])
 def test_tensor_off_the_16_byte_grid(dtype, offset):

@@ -325,9 +325,8 @@ __global__ void __launch_bounds__(1024) k_head_out(HeadOutArgs a) {
 // CTA b < nchunk: the head's pattern of the tail pass, the same for every slab. The entries of a
 // slab, cut into chunks of `chunk` entries, are listed by bucket (sum of the head modes' hashes mod
 // J) within each chunk, in blocks of four 16-bit entry numbers; a bucket's last block is filled up
-// with a number from `chunk` on, an entry that is staged as zero (FP8: there are n_0 of them, and the
-// one of a row that the bucket holds is taken, so that no other row's scale, which may be infinite,
-// enters the sum). Bucket word: first block | blocks << 16.
+// with a number from `chunk` on, an entry that is staged as zero (FP8: there are n_0 of them, one of each
+// row, and the one of a row that the bucket holds is taken). Bucket word: first block | blocks << 16.
 // Sign word: the signs (product of the head modes' v) of 32 entries.
 // CTA nchunk (when R > 0): the slabs of the head pass sorted by c, the hash of the modes 2 .. d-1
 // (plan word: fibre index of the slab | sign << 31). One CTA sorts up to 2^15 slabs; with more the
@@ -510,7 +509,11 @@ __device__ __forceinline__ void add2(unsigned long long& q, unsigned long long x
 // Bound: instruction issue (61% active; 115 M warp instructions) and the random shared-memory loads
 // (150 k of 331 k cycles). 100^4 FP32: 181 us for both modes at J = 4096 (160 us without the copies, one
 // launch per mode 206 us).
-template <int DT, int V, int EPW, int RPT>
+// FP8 scales that are infinite or NaN: the lists' padding, a zero times such a scale, must stay out of the
+// sums. Such tensors take the WILD instance, which skips it entry by entry; both are launched and the CTAs of
+// the one that does not apply return once they have read the scales (3 us; a test in the sums: 13 us of
+// 234 at 40^5).
+template <int DT, int V, int EPW, int RPT, bool WILD = false>
 __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
   using Sh = TailShape<DT, V, EPW>;
   constexpr int EB = Sh::EB, JJ = Sh::JJ, ENT = Sh::ENT, T = TAIL_T;
@@ -523,8 +526,14 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
   float* ssc = reinterpret_cast<float*>(sb + a.J);                                           // n0 FP8 scales
   const int t = threadIdx.x, J = a.J, parts = a.parts;
   const int part = t & (parts - 1), row0 = t / parts, rstep = T / parts;
-  if (DT == TT_FP8E4M3)
-    for (int i = t; i < a.n0; i += T) ssc[i] = __ldg(a.scales + i);
+  if (DT == TT_FP8E4M3) {
+    bool wild = false;
+    for (int i = t; i < a.n0; i += T) {
+      ssc[i] = __ldg(a.scales + i);
+      wild = wild || !isfinite(ssc[i]);
+    }
+    if ((__syncthreads_or(wild) != 0) != WILD) return;
+  }
   for (int i = t; i < zeros * ENT; i += T) buf[(size_t)a.chunk * ENT + i] = 0;
   const int64_t u0 = a.units * blockIdx.x / gridDim.x, u1 = a.units * (blockIdx.x + 1) / gridDim.x;
   if (u0 >= u1) return;
@@ -704,7 +713,10 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
       } else {
         for (int p = p0 + part; p < pe; p += parts) {
           const uint2 x = sl[p];
-          if constexpr (RPT <= 2) {  // buckets of several blocks: each block on its own
+          if constexpr (WILD) {
+            for (uint32_t y : {x.x & 0xFFFFu, x.x >> 16, x.y & 0xFFFFu, x.y >> 16})
+              if (y < (uint32_t)a.chunk) gather(y, q);
+          } else if constexpr (RPT <= 2) {  // buckets of several blocks: each block on its own
             float qb[V] = {};
             gather(x.x & 0xFFFFu, qb);
             gather(x.x >> 16, qb);
@@ -790,6 +802,11 @@ int launch_tail_v(tt_ctx* c, TailArgs a) {
   const int blocks = (int)std::min<int64_t>(a.units, pass_ctas(c, 1));
   kern<<<blocks, TAIL_T, smem, c->stream>>>(a);
   TT_LAUNCH(c, "k_tail_pass");
+  if constexpr (DT == TT_FP8E4M3) {  // (eight buckets per thread hold any J)
+    TT_CUDA(c, cudaFuncSetAttribute(k_tail_pass<DT, V, EPW, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_tail_pass<DT, V, EPW, 8, true><<<blocks, TAIL_T, smem, c->stream>>>(a);
+    TT_LAUNCH(c, "k_tail_pass");
+  }
   return TT_OK;
 }
 

@@ -118,6 +118,30 @@ def test_an_infinite_row_scale_stays_in_its_buckets(row):
     ctx.close()
 
 
+@pytest.mark.parametrize("dims,J", [((32, 24, 7, 5), 4096), ((32, 24, 7, 5), 1024), ((23, 31, 6), 2048)])
+def test_an_infinite_row_scale_keeps_its_sign(dims, J):
+    """FP8 with one infinite scale: a bucket that one non-zero entry of that row falls into holds its signed
+    infinity, whatever else it sums."""
+    seed, row = 977, 13
+    flat, scales, exact = synth.quantize(synth.random_tensor(dims, 31), "fp8")
+    scales = scales.copy()
+    scales[row] = np.inf
+    ctx = lib.Context(dims, [1] + [2] * (len(dims) - 1) + [1], J, 1e-3, seed, "fp8")
+    Y = [torch.empty(n, J, device="cuda") for n in dims]
+    ctx.tt_sketch_unfold(lib.device_tensor(flat, "fp8"), -1, 4, Y, torch.from_numpy(scales).cuda())
+    hs, vs = O.draw_sketch(seed, 4, dims, J)
+    hit, value = np.zeros(dims), np.zeros(dims)
+    hit[row] = 1.0
+    value[row] = exact[row]
+    ones = [np.ones_like(v) for v in vs]
+    for k, n in enumerate(dims):
+        one = np.stack([O.sketch_unfolding_column(hit, hs, ones, J, k, i) for i in range(n)]) == 1
+        val = np.stack([O.sketch_unfolding_column(value, hs, vs, J, k, i) for i in range(n)])
+        one &= val != 0
+        assert one.any() and np.array_equal(Y[k].cpu().numpy()[one], np.copysign(np.inf, val[one])), k
+    ctx.close()
+
+
 def test_more_slabs_than_one_cta_sorts():
     """33,800 slabs of 512 entries: the head pass takes them from mode 1's grid-wide plan."""
     _check((32, 16, 130, 260), 1024, "f32", columns=3)

@@ -892,7 +892,10 @@ bool tail_takes(const tt_ctx* c, const void* A) {
 // Which modes the passes cover, from the shape alone. Workspaces of both sketch draws follow from it.
 // The head pass needs slabs that fill a CTA's warps (512 entries) and columns that leave room for four
 // in a chunk; its row accumulators stay in L2 (32 MB). The tail pass needs chunks of at least that
-// size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. Where the copies
+// size, and a slab that is not much sparser than the J buckets each unit adds to Y_s. With two tail modes
+// every slab costs a unit of its own, so that many small slabs are slower than one launch per mode (4 x 10^6
+// to 10^8 entries: 1.6 and 3 times its time below 1024 entries a slab, 0.12 to 2.3 below 2048, where fibres
+// off the 16-byte grid make the launches slow, 0.7 above): those take no pass. Where the copies
 // of a pass exceed 48 MB each mode takes half as many, and where those do, no pass: with fewer its
 // sums would be off by more than those of one launch per mode. J up to 8192: eight buckets per thread.
 // One row per slab column (n_0 = 1) goes one launch per mode: the passes divide entry numbers by n_0 with a
@@ -931,7 +934,8 @@ void tt_pass_plan(tt_ctx* c) {
       c->tail_blocks = c->tail_chunk / 4 + std::min(c->J, c->tail_chunk);
       fits = tail_smem(c->tail_chunk, c->tail_blocks, c->J, fp8 ? 4 : 8, fp8 ? c->n[0] : 0) <= 227 * 1024;
     }
-    c->pass_tail = fits && E >= 512 && E * 8 >= c->J && c->tail_nchunk <= 64;
+    const bool small = nt == 2 && c->N > 4000000 && (c->n[0] * tt_elem_bytes(c->dtype) % 16 ? E < 1024 : E < 2048);
+    c->pass_tail = fits && E >= 512 && !small && E * 8 >= c->J && c->tail_nchunk <= 64;
     if (c->pass_tail) {
       const int run = tail_run(c->dtype);
       const double slabs = (double)c->tail_nchunk * c->n[c->d - 1];  // that a bucket of Y_s meets

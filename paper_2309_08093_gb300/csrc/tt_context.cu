@@ -820,12 +820,15 @@ extern "C" int tt_sketch_init(tt_ctx** out, const tt_params* p, void* stream) {
   tt_pass_plan(c);
   uint64_t planned = tt_workspace_plan(c);
   const uint64_t cap = g_workspace_limit.load();
-  if (cap && planned > cap && (c->pass_head || c->pass_tail)) {  // one launch per mode needs less
+  auto drop_passes = [&]() {  // one launch per mode needs less; false if there are none to drop
+    if (!c->pass_head && !c->pass_tail) return false;
     c->pass_head = c->pass_tail = c->head_sorted = false;
     c->tail_modes = 0;
     planned = tt_workspace_plan(c);
-  }
-  c->ws_bytes = planned;
+    return true;
+  };
+  // no passes where their workspaces would leave the cap no room for the host-buffer calls' staging
+  if (cap && planned + tt_host_stage_bytes(c) > cap) drop_passes();
   if (cap && planned > cap) {
     fprintf(stderr, "tt_sketch_init: workspaces need %llu bytes, above the limit of %llu bytes\n",
             (unsigned long long)planned, (unsigned long long)cap);
@@ -834,6 +837,11 @@ extern "C" int tt_sketch_init(tt_ctx** out, const tt_params* p, void* stream) {
   }
   // one allocation, cut into the workspaces on 256-byte boundaries as tt_workspace_plan counts them
   cudaError_t e = cudaMalloc(&c->ws_block, planned);
+  if (e == cudaErrorMemoryAllocation && drop_passes()) {
+    cudaGetLastError();  // clear it
+    e = cudaMalloc(&c->ws_block, planned);
+  }
+  c->ws_bytes = planned;
   char* at = static_cast<char*>(c->ws_block);
   if (e == cudaSuccess)
     tt_workspace_each(c, [&](void** ptr, size_t bytes) {

@@ -81,13 +81,17 @@ void tt_host_free(tt_ctx* c) {
 
 static size_t core_bytes(const tt_ctx* c, int k) { return sizeof(float) * (size_t)c->r[k] * c->n[k] * c->r[k + 1]; }
 
+uint64_t tt_host_stage_bytes(const tt_ctx* c) {
+  uint64_t bytes = 2 * ((uint64_t)c->N * tt_elem_bytes(c->dtype) + sizeof(float) * c->n[0]);
+  for (int k = 0; k < c->d; ++k) bytes += core_bytes(c, k);
+  return bytes;
+}
+
 // staging buffers, the copy stream, its events and the pinned result slots, on first use
 static int host_setup(tt_ctx* c, bool scales) {
   const size_t abytes = (size_t)c->N * tt_elem_bytes(c->dtype);
   if (!c->d_A_stage[0]) {  // the staging buffers count against the workspace cap
-    uint64_t extra = 2 * (abytes + sizeof(float) * c->n[0]);
-    for (int k = 0; k < c->d; ++k) extra += core_bytes(c, k);
-    TT_TRY(tt_check_workspace_cap(c, extra));
+    TT_TRY(tt_check_workspace_cap(c, tt_host_stage_bytes(c)));
     for (int b = 0; b < 2; ++b) {
       TT_CUDA(c, cudaMalloc(&c->d_A_stage[b], abytes));
       TT_CUDA(c, cudaEventCreateWithFlags(&c->ev_copied[b], cudaEventDisableTiming));

@@ -266,7 +266,8 @@ struct tt_ctx {
 #define TT_BATCH_ITEM_BYTES (1024 * 1024)
 // bytes of one pinned result slot: the status word, the two error sums, 2 d change sums per sweep
 size_t tt_host_slot_bytes(const tt_ctx* c);
-// the host-buffer calls' resources (tt_host.cu)
+// device bytes of the host-buffer calls' staging buffers; those calls' resources (tt_host.cu)
+uint64_t tt_host_stage_bytes(const tt_ctx* c);
 void tt_host_free(tt_ctx* c);
 
 // ---------------------------------------------------------------------------------------------

@@ -178,6 +178,32 @@ def test_a_workspace_cap_that_leaves_no_room_for_the_passes():
     ctx.close()
 
 
+def test_a_workspace_cap_leaves_room_for_the_host_calls():
+    """The smallest cap under which one launch per mode and the host-buffer calls' staging fit: the passes'
+    workspaces must not take that room."""
+    dims, J, ranks = (40, 36, 30, 9), 64, (1, 2, 2, 2, 1)
+    flat = synth.quantize(synth.random_tensor(dims, 3), "f32")[0]
+    cores = [np.asarray(g, np.float32).ravel(order="F").copy() for g in synth.random_tt(dims, ranks, 4)]
+    stage = 2 * (4 * flat.size + 4 * dims[0]) + sum(4 * g.size for g in cores)
+    lo, hi = 1 << 16, 1 << 26  # smallest cap that still creates a context
+    prev = lib.tt_set_workspace_limit(0)
+    try:
+        while hi - lo > 64:
+            mid = (lo + hi) // 2
+            lib.tt_set_workspace_limit(mid)
+            try:
+                lib.Context(dims, ranks, J, 1e-3, 5).close()
+                hi = mid
+            except lib.TtError:
+                lo = mid
+        lib.tt_set_workspace_limit(hi + stage)
+        ctx = lib.Context(dims, ranks, J, 1e-3, 5)
+        ctx.tt_prox_als_sweep_host(np.ascontiguousarray(flat, np.float32), cores, 1)
+        ctx.close()
+    finally:
+        lib.tt_set_workspace_limit(prev)
+
+
 # Rounding of FP32 sums: n adds one after the other, each off by at most 2^-24 of the partial sum, leave a
 # relative error of at most about 2^-24 sqrt(n / 2) of a sum of n terms of random sign (the partial sums
 # grow with the square root); the levels of a sum (a bucket's entries of one slab, the slabs of one copy,

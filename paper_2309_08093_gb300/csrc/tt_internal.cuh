@@ -378,6 +378,14 @@ int tt_one_sweep(tt_ctx* c, const void* A, const float* scales, float* const* co
 int tt_prof_begin(tt_ctx* c, int k0, int k1);  // record a start event when profiling (returns TT_OK)
 int tt_prof_end(tt_ctx* c);
 int tt_elem_bytes(int dtype);
+// Lets `kern` take the dynamic shared memory an SM has (226 KB: up to 1 KB of static arrays beside it). One
+// value whatever the launch needs, because the attribute belongs to the function: a size per launch would be
+// overwritten between here and the launch by another thread's context of another shape.
+constexpr int TT_SMEM_MAX = 226 * 1024;
+template <typename F>
+cudaError_t tt_allow_smem(F* kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TT_SMEM_MAX);
+}
 // number of SMs of the current device (queried once per device; 152 if the query fails)
 int tt_sm_count();
 // TT_ENOMEM (with a message) when the context's workspaces plus `extra` bytes would exceed the

@@ -798,12 +798,12 @@ int launch_tail_v(tt_ctx* c, TailArgs a) {
                            : a.J <= 2048 ? k_tail_pass<DT, V, EPW, 2>
                            : a.J <= 4096 ? k_tail_pass<DT, V, EPW, 4>
                                          : k_tail_pass<DT, V, EPW, 8>;
-  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TT_CUDA(c, tt_allow_smem(kern));
   const int blocks = (int)std::min<int64_t>(a.units, pass_ctas(c, 1));
   kern<<<blocks, TAIL_T, smem, c->stream>>>(a);
   TT_LAUNCH(c, "k_tail_pass");
   if constexpr (DT == TT_FP8E4M3) {  // (eight buckets per thread hold any J)
-    TT_CUDA(c, cudaFuncSetAttribute(k_tail_pass<DT, V, EPW, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TT_CUDA(c, tt_allow_smem(k_tail_pass<DT, V, EPW, 8, true>));
     k_tail_pass<DT, V, EPW, 8, true><<<blocks, TAIL_T, smem, c->stream>>>(a);
     TT_LAUNCH(c, "k_tail_pass");
   }
@@ -852,7 +852,7 @@ template <int DT, int VB>
 int launch_head_vb(tt_ctx* c, HeadArgs a) {
   const HeadGeom g = head_geom(c);
   auto kern = k_head_pass<DT, VB>;
-  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+  TT_CUDA(c, tt_allow_smem(kern));
   int per_sm = 1;
   TT_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, g.threads, g.smem));
   a.nseg = (int)std::max<int64_t>(1, std::min<int64_t>(a.R, pass_ctas(c, std::min(per_sm, g.per_sm)) / a.nch));
@@ -932,7 +932,7 @@ void tt_pass_plan(tt_ctx* c) {
       c->tail_chunk = (int)((std::min(cm, (E + c->tail_nchunk - 1) / c->tail_nchunk) + 3) & ~3);
       // a bucket's blocks: all full but its last one
       c->tail_blocks = c->tail_chunk / 4 + std::min(c->J, c->tail_chunk);
-      fits = tail_smem(c->tail_chunk, c->tail_blocks, c->J, fp8 ? 4 : 8, fp8 ? c->n[0] : 0) <= 227 * 1024;
+      fits = tail_smem(c->tail_chunk, c->tail_blocks, c->J, fp8 ? 4 : 8, fp8 ? c->n[0] : 0) <= TT_SMEM_MAX;
     }
     const bool small = nt == 2 && c->N > 4000000 && (c->n[0] * tt_elem_bytes(c->dtype) % 16 ? E < 1024 : E < 2048);
     c->pass_tail = fits && E >= 512 && !small && E * 8 >= c->J && c->tail_nchunk <= 64;
@@ -1003,7 +1003,7 @@ int tt_launch_pass_plans(tt_ctx* c) {
   p.nkeys = (int)((std::max<int64_t>(p.nchunk ? p.chunk : 0, p.R) + 3) & ~3);
   const size_t smem = sizeof(int) * (size_t)((c->J + 1) & ~1) +
                       sizeof(uint16_t) * (p.nkeys + std::max<size_t>(p.nchunk ? 4 * (size_t)p.blocks : 0, p.R));
-  TT_CUDA(c, cudaFuncSetAttribute(k_pass_plans, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TT_CUDA(c, tt_allow_smem(k_pass_plans));
   k_pass_plans<<<ctas, 1024, smem, c->stream>>>(p);
   TT_LAUNCH(c, "k_pass_plans");
   return TT_OK;

@@ -437,15 +437,13 @@ __global__ void __launch_bounds__(QT, 1) k_lq_tiles(LqArgs a, const int* status)
   }
 }
 
-constexpr size_t SMEM_MAX = 227 * 1024;
-
 template <int Q>
 bool launch_left(tt_ctx* c, float* core, float* next, int r0, int n, int q, int ncols, cudaError_t* err) {
   const int64_t m = (int64_t)r0 * n, nx = (int64_t)q * ncols;
-  const int prefetch = qr_smem<Q>(m, nx) <= SMEM_MAX;
+  const int prefetch = qr_smem<Q>(m, nx) <= TT_SMEM_MAX;
   const size_t smem = qr_smem<Q>(m, prefetch ? nx : 0);
-  if (smem > SMEM_MAX) return false;
-  *err = cudaFuncSetAttribute(k_qr_left_tiles<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > TT_SMEM_MAX) return false;
+  *err = tt_allow_smem(k_qr_left_tiles<Q>);
   if (*err != cudaSuccess) return true;
   k_qr_left_tiles<Q><<<1, QT, smem, c->stream>>>(core, next, r0, n, q, ncols, prefetch, c->d_status);
   *err = cudaGetLastError();
@@ -454,10 +452,10 @@ bool launch_left(tt_ctx* c, float* core, float* next, int r0, int n, int q, int 
 
 template <int Q>
 bool launch_lq(tt_ctx* c, LqArgs a, cudaError_t* err) {
-  if (qr_smem<Q>(a.mmax, a.nxmax) > SMEM_MAX) a.nxmax = 0;
+  if (qr_smem<Q>(a.mmax, a.nxmax) > TT_SMEM_MAX) a.nxmax = 0;
   const size_t smem = qr_smem<Q>(a.mmax, a.nxmax);
-  if (smem > SMEM_MAX) return false;
-  *err = cudaFuncSetAttribute(k_lq_tiles<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > TT_SMEM_MAX) return false;
+  *err = tt_allow_smem(k_lq_tiles<Q>);
   if (*err != cudaSuccess) return true;
   k_lq_tiles<Q><<<1, QT, smem, c->stream>>>(a, c->d_status);
   *err = cudaGetLastError();

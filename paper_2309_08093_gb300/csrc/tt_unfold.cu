@@ -93,7 +93,7 @@ static int launch_cols_s(tt_ctx* c, const void* A, const float* scales, int k, f
     if constexpr (4 * EPV <= 16)
       if (mv == 4) kern = k_unfold_cols<DT, VB, S, 4, G>;
   }
-  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TT_CUDA(c, tt_allow_smem(kern));
   const int items = ncolg * a.nseg;
   kern<<<std::max(1, items), THREADS, smem, c->stream>>>(a);
   TT_LAUNCH(c, "k_unfold_cols");
@@ -154,7 +154,7 @@ static int launch_gather_vbm(tt_ctx* c, const void* A, const float* scales, int 
   // to leave (measured at 100^4: -5% per step). Not in graph capture, where other tensors share
   // the SMs.
   const size_t smem_l = ONE_CTA ? std::max(smem, (size_t)116 * 1024) : smem;
-  TT_CUDA(c, cudaFuncSetAttribute(k_unfold_gather<DT, VB, S, M, MODE0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_l));
+  TT_CUDA(c, tt_allow_smem(k_unfold_gather<DT, VB, S, M, MODE0>));
   int per_sm = 1;
   TT_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_unfold_gather<DT, VB, S, M, MODE0>, THREADS, smem));
   const int items = a.ncol * a.nseg;

@@ -423,7 +423,7 @@ int win_nseg(tt_ctx* c, int k, int units, int slots) {
 template <int DT, int S, int EPT>
 int cols_win_launch(tt_ctx* c, const GArgs& a, size_t smem, int blocks) {
   auto kern = k_unfold_cols_win<DT, S, EPT>;
-  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TT_CUDA(c, tt_allow_smem(kern));
   kern<<<blocks, WIN_THREADS, smem, c->stream>>>(a);
   TT_LAUNCH(c, "k_unfold_cols_win");
   return TT_OK;
@@ -483,7 +483,7 @@ int gather_win_launch(tt_ctx* c, const void* A, const float* scales, int k, floa
   *done = true;
   TT_CUDA(c, cudaMemsetAsync(Y, 0, sizeof(float) * c->J * c->n[k], c->stream));  // empty groups stay 0
   auto kern = k_unfold_gather_win<DT, S, LPF, EPT, MODE0>;
-  TT_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TT_CUDA(c, tt_allow_smem(kern));
   int per_sm = 1;
   TT_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WIN_THREADS, smem));
   const int items = a.ncol * a.nseg;

@@ -5,6 +5,8 @@ chunks (10,240 entries; 5,120 in FP64), chunks that end inside a column, slabs o
 1-byte boundaries, odd groups of tail indices, sketch sizes from fewer buckets than a CTA's threads
 share up to 8192, more slabs than one CTA sorts, and tensors that start off the 16-byte grid. The
 tolerance is the suite's for FP32 sums (1e-5 relative)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -202,6 +204,43 @@ def test_a_workspace_cap_leaves_room_for_the_host_calls():
         ctx.close()
     finally:
         lib.tt_set_workspace_limit(prev)
+
+
+def test_contexts_of_different_shapes_in_threads():
+    """Contexts whose launches of one kernel need different amounts of shared memory, each driven by a thread
+    of its own: every call succeeds, and the sketches are those of calls from one thread."""
+    shapes = [((20, 30, 6, 5), 64), ((100, 100, 4, 3), 1024), ((40, 16, 6, 5), 128), ((100, 90, 4, 3), 1000)]
+    work = []
+    for dims, J in shapes:
+        ctx = lib.Context(dims, (1, 2, 2, 2, 1), J, 1e-3, 5)
+        A = lib.device_tensor(synth.quantize(synth.random_tensor(dims, 3), "f32")[0], "f32")
+        Y = [[torch.empty(n, J, device="cuda") for n in dims] for _ in range(2)]
+        ctx.tt_sketch_unfold(A, -1, 0, Y[0])
+        work.append((ctx, A, Y))
+    torch.cuda.synchronize()
+    errors, start = [], threading.Barrier(len(work))
+
+    def drive(ctx, A, Y):
+        start.wait()
+        try:
+            for t in range(400):
+                ctx.tt_sketch_unfold(A, -1, t % 2, Y[1])  # two draws in turn: plans too
+                ctx.tt_sketch_unfold(A, t % 4, t % 2, Y[1])
+            ctx.tt_sketch_unfold(A, -1, 0, Y[1])
+        except lib.TtError as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=drive, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors[0]
+    for ctx, _, Y in work:
+        for a, b in zip(*Y):
+            assert float(torch.linalg.vector_norm(a - b)) <= TOL * float(torch.linalg.vector_norm(a))
+        ctx.close()
 
 
 # Rounding of FP32 sums: n adds one after the other, each off by at most 2^-24 of the partial sum, leave a

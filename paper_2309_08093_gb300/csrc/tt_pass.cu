@@ -85,21 +85,22 @@ __device__ __forceinline__ int tile_at(int i1, int i0, int pitch) {
   return i1 * pitch + ((((i0 >> 2) ^ ((i1 >> 2) & 7)) << 2) | (i0 & 3));
 }
 
-// VB bytes of A as 32-bit words
+// VB bytes of A as 32-bit words. A is read with the streaming hint here and in the tail pass, so that the
+// accumulators' copies stay in L2 beside it (100^4 FP32, all modes: 308 -> 297 us).
 template <int VB>
 __device__ __forceinline__ void head_load(const char* p, uint32_t* r) {
   if constexpr (VB == 16) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint4 u = __ldcs(reinterpret_cast<const uint4*>(p));
     r[0] = u.x, r[1] = u.y, r[2] = u.z, r[3] = u.w;
   } else if constexpr (VB == 8) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 u = __ldcs(reinterpret_cast<const uint2*>(p));
     r[0] = u.x, r[1] = u.y;
   } else if constexpr (VB == 4) {
-    r[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+    r[0] = __ldcs(reinterpret_cast<const uint32_t*>(p));
   } else if constexpr (VB == 2) {
-    r[0] = __ldg(reinterpret_cast<const unsigned short*>(p));
+    r[0] = __ldcs(reinterpret_cast<const unsigned short*>(p));
   } else {
-    r[0] = __ldg(reinterpret_cast<const unsigned char*>(p));
+    r[0] = __ldcs(reinterpret_cast<const unsigned char*>(p));
   }
 }
 
@@ -140,9 +141,9 @@ __device__ __forceinline__ void head_add(const uint32_t* w, float s, float* acc)
   }
 }
 
-// Bound: DRAM while runs are long (100^4 FP32, J = 1024, 9.8 slabs per run: 98 us with k_head_out, 170 us
+// Bound: DRAM while runs are long (100^4 FP32, J = 1024, 9.8 slabs per run: 80 us with k_head_out, 170 us
 // with one launch per mode), the flushes' L2 atomics and tile traffic beside it when they are short
-// (J = 4096, 2.4 slabs per run: 132 and 206 us). The flushes go to L2 as 16-byte atomic adds
+// (J = 4096, 2.4 slabs per run: 128 and 206 us). The flushes go to L2 as 16-byte atomic adds
 // along rows (5.9 TB/s of sums, measured alone) because shared-memory float atomics at random
 // buckets sustain half of that (0.75 T adds/s) and need a copy of the columns per CTA. Two CTAs per
 // SM: one flushes while the other loads.
@@ -507,7 +508,7 @@ __device__ __forceinline__ void add2(unsigned long long& q, unsigned long long x
 // one launch per mode: 256 x 256 x 3 x 128 FP32 5.4e-7 / 1.1e-7 / 2.0e-7, 40^5 FP8 2.2e-7 / 7.3e-8 /
 // 7.8e-8, 100^4 FP32 1.8e-7 / 7.9e-8 / 9.5e-8.
 // Bound: instruction issue (61% active; 115 M warp instructions) and the random shared-memory loads
-// (150 k of 331 k cycles). 100^4 FP32: 181 us for both modes at J = 4096 (160 us without the copies, one
+// (150 k of 331 k cycles). 100^4 FP32: 176 us for both modes at J = 4096 (161 us without the copies, one
 // launch per mode 206 us).
 // FP8 scales that are infinite or NaN: the lists' padding, a zero times such a scale, must stay out of the
 // sums. Such tensors take the WILD instance, which skips it entry by entry; both are launched and the CTAs of
@@ -553,10 +554,10 @@ __global__ void __launch_bounds__(TAIL_T, 1) k_tail_pass(TailArgs a) {
       for (int jj = 0; jj < JJ; ++jj) {
         if (jj < nj) {
           const char* q = p + T * jj * (EPW * EB);
-          if constexpr (EPW * EB == 8) pw[jj][v] = __ldg(reinterpret_cast<const double*>(q));
-          else if constexpr (EPW * EB == 4) pw[jj][v] = __ldg(reinterpret_cast<const uint32_t*>(q));
-          else if constexpr (EPW * EB == 2) pw[jj][v] = __ldg(reinterpret_cast<const unsigned short*>(q));
-          else pw[jj][v] = __ldg(reinterpret_cast<const unsigned char*>(q));
+          if constexpr (EPW * EB == 8) pw[jj][v] = __ldcs(reinterpret_cast<const double*>(q));
+          else if constexpr (EPW * EB == 4) pw[jj][v] = __ldcs(reinterpret_cast<const uint32_t*>(q));
+          else if constexpr (EPW * EB == 2) pw[jj][v] = __ldcs(reinterpret_cast<const unsigned short*>(q));
+          else pw[jj][v] = __ldcs(reinterpret_cast<const unsigned char*>(q));
         }
       }
     }

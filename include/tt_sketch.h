@@ -112,7 +112,10 @@ typedef struct {
 /*
  * Create a context for tensors of the given shape (Alg. 1 inputs: A's shape, TT ranks,
  * sketch size m, sigma). `cuda_stream` is a cudaStream_t (NULL = legacy default stream).
- * Allocates all device workspaces. Returns TT_EINVAL for inconsistent parameters.
+ * Allocates all device workspaces, those of the all-modes data sketches too (accumulators of at most
+ * 96 MB and plans: a context of a 100^4 FP32 tensor at J = 4096 owns 114 MB, 72 MB without them; they
+ * are left out where a cap or the device has no room for them). Returns TT_EINVAL for inconsistent
+ * parameters.
  */
 int tt_sketch_init(tt_ctx** out, const tt_params* p, void* cuda_stream);
 
@@ -127,7 +130,8 @@ const char* tt_last_error(const tt_ctx* ctx);
  * the previous cap. The paper has no counterpart: it is memory budgeting for applications that
  * share the GPU. tt_sketch_init sums the sizes of all the workspaces it would allocate (hash
  * tables, fibre plans of two draws, FFT sketches, data sketches, Gram and solve buffers, the
- * relative error's interfaces) before any CUDA call, and returns TT_ENOMEM (message on stderr)
+ * relative error's interfaces; the all-modes sketches' workspaces only where the cap then still holds
+ * tt_prox_als_sweep_host's staging buffers) before any CUDA call, and returns TT_ENOMEM (message on stderr)
  * when the sum exceeds the cap; tt_prox_als_sweep_host returns TT_ENOMEM the same way before it
  * allocates its staging buffers (the tensor, the scales and the cores) beyond the cap. Contexts
  * created before a change keep what they own. Thread-safe.

@@ -507,8 +507,8 @@ __device__ __forceinline__ void add2(unsigned long long& q, unsigned long long x
 // lists are summed block by block where a bucket has several. Relative error of Y_s, one sum / in levels /
 // one launch per mode: 256 x 256 x 3 x 128 FP32 5.4e-7 / 1.1e-7 / 2.0e-7, 40^5 FP8 2.2e-7 / 7.3e-8 /
 // 7.8e-8, 100^4 FP32 1.8e-7 / 7.9e-8 / 9.5e-8.
-// Bound: instruction issue (61% active; 115 M warp instructions) and the random shared-memory loads
-// (150 k of 331 k cycles). 100^4 FP32: 176 us for both modes at J = 4096 (161 us without the copies, one
+// Bound: instruction issue (64% active; 123 M warp instructions) and the random shared-memory loads
+// (141 k of 333 k cycles). 100^4 FP32: 176 us for both modes at J = 4096 (161 us without the copies, one
 // launch per mode 206 us).
 // FP8 scales that are infinite or NaN: the lists' padding, a zero times such a scale, must stay out of the
 // sums. Such tensors take the WILD instance, which skips it entry by entry; both are launched and the CTAs of

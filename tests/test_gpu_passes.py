@@ -144,6 +144,12 @@ def test_an_infinite_row_scale_keeps_its_sign(dims, J):
     ctx.close()
 
 
+@pytest.mark.parametrize("slabs", [40, 120, 240])
+def test_accumulators_near_their_bound(slabs):
+    """700 x 300 slabs at J = 8192: a head pass with the copies its sums ask for, with half of them, and none."""
+    _check((700, 300, slabs), 8192, "f32", columns=3, rank=1)
+
+
 def test_more_slabs_than_one_cta_sorts():
     """33,800 slabs of 512 entries: the head pass takes them from mode 1's grid-wide plan."""
     _check((32, 16, 130, 260), 1024, "f32", columns=3)
